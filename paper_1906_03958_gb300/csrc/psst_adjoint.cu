@@ -80,16 +80,6 @@ __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ float ratio_u_deriv(float u) {
-    // d/du of u / (1 - e^{-u}); Bernoulli series near 0
-    if (fabsf(u) < 0.1f) {
-        const float u2 = u * u;
-        return fmaf(u, fmaf(u2, -1.0f / 180.0f, 1.0f / 6.0f), 0.5f);
-    }
-    const float e = expf(-u), den = -expm1f(-u);
-    return __fdiv_rn(den - u * e, den * den);
-}
-
 struct AdjSmem {
     // forward CTA: row items (row-aligned, K chunks of 4 synapses,
     // slot-major) with the pair of each synapse in id; sweeping CTA: column
@@ -177,7 +167,7 @@ __device__ void fwd_step(const NetView &v, const AdjNet &a, const AdjSmem &S, co
         S.sn[i] = n[i];
         for (int t = 0; t < nt; ++t) {
             const int p = i * nt + t;
-            const float *sp = stab + t * 9;
+            const float *sp = stab + t * ST_COLS;
             S.sr[p] = r[p];
             S.ss[p] = s[p];
             const float s2 = s[p] * s[p], s4 = s2 * s2;
@@ -267,10 +257,10 @@ __device__ void fwd_step(const NetView &v, const AdjNet &a, const AdjSmem &S, co
             } else {
                 // gate pair p = (presynaptic neuron i, type t)
                 const int p = u - 2 * N, i = p / nt, t = p - i * nt;
-                const float *sp = stab + t * 9;
+                const float *sp = stab + t * ST_COLS;
                 const float Vs = S.sV[st * N + i];
                 const float rs = S.sr[st * M + p], ss = S.ss[st * M + p];
-                const float T = transmitter(Vs, sp[SP_VP], sp[SP_KP]);
+                const float T = transmitter(Vs, sp);
                 const float dr = sp[SP_A] * T * (1.0f - rs) - sp[SP_B] * rs;
                 const float ds = sp[SP_KIND] != 0.0f ? sp[SP_K3] * rs - sp[SP_K4] * ss : 0.0f;
                 const int ir = 4 * N + p, is = 4 * N + M + p;
@@ -371,24 +361,27 @@ __device__ void rev_step(const AdjNet &a, const AdjSmem &S, const float *stab, c
                 const int ix = x * N + i;
                 const float kbx = cb[st] * S.lam[ix] + (st < NST - 1 ? ca[st] * S.yprev[ix] : 0.0f);
                 float al, be, dal, dbe, g, yp;
+                const float e = rate_e(Vs);
                 if (x == 1) {
-                    al = ratio_u((Vs + 40.0f) * 0.1f);
-                    be = 4.0f * expf((Vs + 65.0f) * (-1.0f / 18.0f));
-                    dal = 0.1f * ratio_u_deriv((Vs + 40.0f) * 0.1f);
+                    const float u = __fmul_rn(__fadd_rn(Vs, 40.0f), 0.1f);
+                    al = alpha_m(Vs, e);
+                    be = beta_m(Vs);
+                    dal = 0.1f * ratio_u_deriv(u, al, e, __fsub_rn(1.0f, e));
                     dbe = -be * (1.0f / 18.0f);
                     g = ms;
                     yp = -q * gNa * 3.0f * ms * ms * hs * (Vs - ENa);
                 } else if (x == 2) {
-                    al = 0.07f * expf((Vs + 65.0f) * (-1.0f / 20.0f));
-                    be = __frcp_rn(1.0f + expf((Vs + 35.0f) * (-0.1f)));
+                    al = alpha_h(Vs);
+                    be = beta_h(e);
                     dal = -al * (1.0f / 20.0f);
                     dbe = be * (1.0f - be) * 0.1f;
                     g = hs;
                     yp = -q * gNa * ms * ms * ms * (Vs - ENa);
                 } else {
-                    al = 0.1f * ratio_u((Vs + 55.0f) * 0.1f);
-                    be = 0.125f * expf((Vs + 65.0f) * (-1.0f / 80.0f));
-                    dal = 0.01f * ratio_u_deriv((Vs + 55.0f) * 0.1f);
+                    const float u = __fmul_rn(__fadd_rn(Vs, 55.0f), 0.1f), den = den_n(e);
+                    al = alpha_n(Vs, e);
+                    be = beta_n(Vs);
+                    dal = 0.01f * ratio_u_deriv(u, 10.0f * al, __fsub_rn(1.0f, den), den);
                     dbe = -be * (1.0f / 80.0f);
                     g = ns;
                     yp = -q * gK * 4.0f * ns * ns * ns * (Vs - EK);
@@ -407,15 +400,15 @@ __device__ void rev_step(const AdjNet &a, const AdjSmem &S, const float *stab, c
         for (int p = tid; p < M; p += nthr) {
             const int i = p / nt, t = p - i * nt;
             const float Vs = S.sV[st * N + i];
-            const float *sp = stab + t * 9;
+            const float *sp = stab + t * ST_COLS;
             float C = 0.0f;  // the pair's column sum: its items' partials in item order
             for (int q = S.ib[p]; q < S.ib[p + 1]; ++q) C += S.pa[q];
             const int ir = 4 * N + p, is = 4 * N + M + p;
             const float kbr = cb[st] * S.lam[ir] + (st < NST - 1 ? ca[st] * S.yprev[ir] : 0.0f);
             const float kbs = cb[st] * S.lam[is] + (st < NST - 1 ? ca[st] * S.yprev[is] : 0.0f);
             const float rs = S.sr[st * M + p], ss = S.ss[st * M + p];
-            const float T = transmitter(Vs, sp[SP_VP], sp[SP_KP]);
-            const float dT = T * (1.0f - T) * sp[SP_KP];  // table holds 1/Kp
+            const float T = transmitter(Vs, sp);
+            const float dT = T * (1.0f - T) * (sp[SP_KP] * 0.693147181f);
             float ur = -(sp[SP_A] * T + sp[SP_B]) * kbr, us = 0.0f;
             if (sp[SP_KIND] != 0.0f) {
                 const float s2 = ss * ss, s4 = s2 * s2, den = s4 + sp[SP_KD];
@@ -579,13 +572,9 @@ __device__ void copy_stages(float *stages, float *blk, int N, int M, int nst) {
 template <int NST, bool TAB>
 __global__ void __launch_bounds__(ADJ_THREADS) adj_kernel(NetView v, AdjView av, long long step0, int nsteps) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ float stab[PSST_MAX_SYN_TYPES * PSST_SYN_NPARAM];
+    __shared__ float stab[PSST_MAX_SYN_TYPES * ST_COLS];
     __shared__ int s_bad;
-    for (int i = threadIdx.x; i < v.n_stypes * PSST_SYN_NPARAM; i += blockDim.x) {
-        float x = v.sparams[i];
-        if (i % PSST_SYN_NPARAM == SP_KP) x = 1.0f / x;
-        stab[i] = x;
-    }
+    load_syn_table(v.sparams, v.n_stypes, stab);
     if (threadIdx.x == 0) s_bad = 0;
     __syncthreads();
     const int tid = threadIdx.x, nthr = blockDim.x;
@@ -655,7 +644,7 @@ __global__ void __launch_bounds__(ADJ_THREADS) adj_kernel(NetView v, AdjView av,
         for (int x = 0; x < 9; ++x) S.gp[9 * i + x] = make_float2(0.0f, 0.0f);
         S.uV[i] = 0.0f;
     }
-    for (int q = tid; q < M; q += nthr) S.Ep[q] = stab[(q % nt) * 9 + SP_E];
+    for (int q = tid; q < M; q += nthr) S.Ep[q] = stab[(q % nt) * ST_COLS + SP_E];
     for (int q = tid; q < a.R; q += nthr) {
         S.lam[q] = 0.0f;
         S.ysum[q] = 0.0f;

@@ -133,7 +133,7 @@ __device__ __forceinline__ void stage(const NetView &v, const SG &sg, const Item
             float4 &f2 = HAS2 ? fin2[p] : d4;
             // presynaptic neuron and synapse type of the entry
             const int pre = PAIR ? (int)(pof[p] >> 8) : p / nt, tp = PAIR ? (int)(pof[p] & 255u) : p % nt;
-            const float *sp = stab + tp * 9;
+            const float *sp = stab + tp * ST_COLS;
             coef_update<HAS2>(sp, vcur[pre], sg, cur1[p], acc1[p], fin1[p], c2, a2, f2);
             if (PAIR) {
                 // the pair's gate for the next stage (same operations as the per-synapse path)
@@ -224,7 +224,7 @@ __device__ void run_net(const NetView &v, int b, const NetPlan &pl, long long st
         fin1[k] = make_float2(0.0f, 0.0f);  // identity maps (increment form)
         if (HAS2) {
             const int ci = PAIR ? v.pair_of[v.pair_off[b] + k] : k;
-            const float *sp = stab + (ci % nt) * 9;
+            const float *sp = stab + (ci % nt) * ST_COLS;
             fin2[k] = make_float4(0.0f, 0.0f, 0.0f, sp[SP_KIND] != 0.0f ? sp[SP_KD] : 1.0f);
         }
     }
@@ -245,7 +245,7 @@ __device__ void run_net(const NetView &v, int b, const NetPlan &pl, long long st
         }
         __syncthreads();
         for (int p = tid; p < M; p += nthr) {
-            const bool sec = HAS2 && stab[(pof[p] & 255u) * 9 + SP_KIND] != 0.0f;
+            const bool sec = HAS2 && stab[(pof[p] & 255u) * ST_COLS + SP_KIND] != 0.0f;
             put_gate(Gt, p, lrep,
                      pair_gate(sec, fin1[p], HAS2 ? fin2[p] : make_float4(0.f, 0.f, 0.f, 1.f), pst[p], pst[M + p],
                                pst[2 * M + p], pst[3 * M + p]));
@@ -322,12 +322,8 @@ template <int CL>
 __global__ void __launch_bounds__(1024) net_kernel(NetView v, const int *list, const NetPlan *plans,
                                                    long long step0, int nsteps, int lrep_cap) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ float stab[PSST_MAX_SYN_TYPES * PSST_SYN_NPARAM];
-    for (int i = threadIdx.x; i < v.n_stypes * PSST_SYN_NPARAM; i += blockDim.x) {
-        float x = v.sparams[i];
-        if (i % PSST_SYN_NPARAM == SP_KP) x = 1.0f / x;  // stored as 1/Kp
-        stab[i] = x;
-    }
+    __shared__ float stab[PSST_MAX_SYN_TYPES * ST_COLS];
+    load_syn_table(v.sparams, v.n_stypes, stab);
     __syncthreads();
     const int b = list[blockIdx.x / CL];
     const uint8_t f = v.net_flags[b];
@@ -394,7 +390,7 @@ cudaError_t pair_check(const NetView &v, uint8_t *out, int smem, cudaStream_t st
     return cudaGetLastError();
 }
 
-int cta_static_smem() { return (int)(PSST_MAX_SYN_TYPES * PSST_SYN_NPARAM * sizeof(float)); }
+int cta_static_smem() { return (int)(PSST_MAX_SYN_TYPES * ST_COLS * sizeof(float)); }
 
 cudaError_t cta_prepare(int cl, int max_smem) {
     const void *k = cl == 1 ? (const void *)net_kernel<1> : cl == 2 ? (const void *)net_kernel<2>

@@ -253,7 +253,7 @@ __device__ __forceinline__ bool grid_stage(const NetView &v, const GridView &g, 
                 float4 f2 = make_float4(0.f, 0.f, 0.f, 0.f), d4 = f2;
                 float4 &c2 = HAS2 ? cur2[p] : d4;
                 float4 &a2 = HAS2 ? acc2[p] : d4;
-                const float *sp = stab + (p % nt) * 9;
+                const float *sp = stab + (p % nt) * ST_COLS;
                 coef_update<HAS2>(sp, vcur[p / nt], sg, cur1[p], acc1[p], f1, c2, a2, f2);
                 const bool sec = HAS2 && sp[SP_KIND] != 0.0f;
                 float G;
@@ -277,7 +277,7 @@ __device__ __forceinline__ bool grid_stage(const NetView &v, const GridView &g, 
                 float4 f2 = make_float4(0.f, 0.f, 0.f, 0.f), d4 = f2;
                 float4 &c2 = HAS2 ? cur2[p] : d4;
                 float4 &a2 = HAS2 ? acc2[p] : d4;
-                coef_update<HAS2>(stab + (p % nt) * 9, vcur[p / nt], sg, cur1[p], acc1[p], f1, c2, a2, f2);
+                coef_update<HAS2>(stab + (p % nt) * ST_COLS, vcur[p / nt], sg, cur1[p], acc1[p], f1, c2, a2, f2);
                 o1[p] = LAST ? f1 : cur1[p];
                 if (HAS2) o2[p] = LAST ? f2 : cur2[p];
             }
@@ -356,7 +356,7 @@ __device__ void grid_run(const NetView &v, const GridView &g, long long step0, i
             const int t = g.tix[(size_t)lo * nt + p];
             float r0 = 0.0f, s0 = 0.0f, rl = 0.0f, sl = 0.0f;
             if (t >= 0) {
-                const float *sp = stab + (p % nt) * 9;
+                const float *sp = stab + (p % nt) * ST_COLS;
                 const bool sec = HAS2 && sp[SP_KIND] != 0.0f;
                 const long long k = g.rep[t];
                 r0 = gr[k];
@@ -381,7 +381,7 @@ __device__ void grid_run(const NetView &v, const GridView &g, long long step0, i
             const int gi = lo * nt + p;
             g.c1[gi] = make_float2(0.0f, 0.0f);  // identity maps (increment form)
             if (HAS2) {
-                const float *sp = stab + (p % nt) * 9;
+                const float *sp = stab + (p % nt) * ST_COLS;
                 g.c2[gi] = make_float4(0.0f, 0.0f, 0.0f, sp[SP_KIND] != 0.0f ? sp[SP_KD] : 1.0f);
             }
         }
@@ -498,14 +498,10 @@ __device__ void grid_run(const NetView &v, const GridView &g, long long step0, i
 
 __global__ void __launch_bounds__(1024, 1) grid_kernel(NetView v, GridView g, long long step0, int nsteps) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ float stab[PSST_MAX_SYN_TYPES * PSST_SYN_NPARAM];
+    __shared__ float stab[PSST_MAX_SYN_TYPES * ST_COLS];
     __shared__ int s_fail;  // set by any thread whose wait failed
     if (threadIdx.x == 0) s_fail = 0;
-    for (int i = threadIdx.x; i < v.n_stypes * PSST_SYN_NPARAM; i += blockDim.x) {
-        float x = v.sparams[i];
-        if (i % PSST_SYN_NPARAM == SP_KP) x = 1.0f / x;
-        stab[i] = x;
-    }
+    load_syn_table(v.sparams, v.n_stypes, stab);
     __syncthreads();
     const bool has2 = v.net_flags[0] & NET_HAS2;
     if (g.pair) {

@@ -104,7 +104,7 @@ __device__ __forceinline__ long long item_slot(int ib, int m, int K, int n, int 
 }
 
 __device__ __forceinline__ bool second_order(const float *stab, uint32_t code) {
-    return stab[(code >> 24) * 9 + SP_KIND] != 0.0f;
+    return stab[(code >> 24) * ST_COLS + SP_KIND] != 0.0f;
 }
 
 // Fill the items of rows [row0, row0 + nrows) of a network from the global
@@ -151,7 +151,7 @@ __device__ void load_items(Items &it, const NetView &v, long long row_g0, long l
             const float w = gw[k];
             R[p] = gr[k];
             W[p] = w;
-            WE[p] = w * stab[(code >> 24) * 9 + SP_E];
+            WE[p] = w * stab[(code >> 24) * ST_COLS + SP_E];
             ID[p] = (unsigned short)(code & 0xFFFFFFu);
             if (HAS2 && sec) Sg[p] = gs[k];
         }
@@ -424,7 +424,7 @@ __device__ inline void load_items_pair(Items &it, const NetView &v, long long ro
         for (int t = 0; t < nt; ++t) {
             base[t] = b;
             const int q = part_items(cnt[t], K);
-            for (int u = 0; u < q; ++u) it.pb[b + u] = stab[t * 9 + SP_E];
+            for (int u = 0; u < q; ++u) it.pb[b + u] = stab[t * ST_COLS + SP_E];
             b += q;
         }
         for (long long k = k0; k < k1; ++k) {
@@ -552,7 +552,7 @@ __device__ __forceinline__ void coef_update(const float *sp, float V, const SG &
                                             float2 &fin, float4 &cur2, float4 &acc2, float4 &fin2) {
     const bool FIRST = sg.first, LAST = sg.last;
     const float WGT = sg.c.w, cnext = sg.c.cn, dt6 = sg.c.fin;
-    const float T = transmitter(V, sp[SP_VP], sp[SP_KP]);  // table holds 1/Kp
+    const float T = transmitter(V, sp);
     // explicit roundings: no product is contracted into an FMA or folded
     // with a constant stage weight, so every kernel and stage kind (constant
     // or run-time coefficients) gets the same bits
