@@ -118,7 +118,11 @@ typedef struct {
     int64_t rec_capacity;          /* frames in the record ring buffer (>= 1 if stride > 0) */
     int32_t mode;                  /* PSST_MODE_* */
     int32_t block_threads;         /* CTA size (multiple of 32, <= 1024), 0 = tuned */
-    int32_t item_chunks;           /* 4-synapse chunks per work item of the synaptic sum (1..64), 0 = tuned */
+    int32_t item_chunks;           /* 4-synapse chunks per work item of the synaptic sum (1..64), 0 = tuned.
+                                      CTA mode with block_threads and item_chunks both 0 holds the synapses of
+                                      per-pair networks (gate_mode) as dense rows instead of work items where
+                                      they fit and no row has two synapses of one (presynaptic neuron, type)
+                                      pair; the two agree to rounding */
     int32_t device;                /* CUDA device ordinal, -1 = current device */
     int32_t gate_mode;             /* 0: one gate per (presynaptic neuron, type) pair whenever all
                                       its synapses' gates are equal (bitwise-identical results,
@@ -126,8 +130,8 @@ typedef struct {
     int32_t method;                /* PSST_METHOD_RK4 (0), PSST_METHOD_EULER (1) or PSST_METHOD_TABLEAU (2) */
     int32_t min_cluster;           /* CTA mode: spread every network of at least 2 x min_cluster neurons
                                       over a cluster of at least min_cluster CTAs (1, 2 or 4; same
-                                      results, shorter steps when SMs are idle); 0 = chosen by
-                                      psst_autotune (default 1) */
+                                      results, shorter steps when SMs are idle); 0 = chosen by the
+                                      library and by psst_autotune */
     int32_t rk_stages;             /* PSST_METHOD_TABLEAU: stages (1..4); ignored otherwise */
     float rk_a[3];                 /* a_2, a_3, a_4: stage s+1 starts at y + dt a_{s+1} k_s (finite) */
     float rk_b[4];                 /* b_1 .. b_{rk_stages}: weights of the step (finite, not all 0) */
@@ -138,7 +142,7 @@ typedef struct {
     int64_t n_neurons, n_synapses;
     int64_t steps_done;            /* global step index of the current state */
     int64_t rec_frames;            /* frames recorded so far (all calls) */
-    int32_t mode, block_threads, item_chunks; /* CTA size and work-item chunks of the last class */
+    int32_t mode, block_threads, item_chunks; /* CTA size and work-item chunks (0: dense rows) of the last class */
     int32_t grid_ctas;             /* CTAs of one integrate chunk (all launches) */
     int32_t smem_bytes;            /* largest dynamic shared memory per CTA */
     int32_t n_single_cta_nets;     /* CTA mode: networks held by one CTA */
@@ -214,7 +218,8 @@ int psst_set_graph_mode(psst_net *h, int enable);
    size class of a CTA-mode handle, time trial_steps steps with twice, once,
    half and a quarter of the class's default CTA size, each with the planned
    number of shared-memory copies of the per-pair gate table and with a
-   single copy, and keep the fastest.  Trials start from a copy of the state
+   single copy (classes of dense rows: the kernel variants that fit, with
+   several CTA sizes), and keep the fastest.  Trials start from a copy of the state
    with recording off; the state is restored.  No choice changes the
    summation order (a larger cluster keeps the work-item size of one CTA),
    so results stay bitwise identical.  Synchronises `stream`.  Grid mode:

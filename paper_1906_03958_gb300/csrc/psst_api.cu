@@ -8,7 +8,9 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "../../include/psst.h"
@@ -67,6 +69,10 @@ struct PlanInput {
     std::vector<int> net_off, n1, n2;
     std::vector<int> tcnt;       // [N][nt] synapses of each type per row
     std::vector<int> pair_off;   // [n_nets + 1] used (presynaptic neuron, type) pairs of the networks
+    std::vector<int> pair_of;    // [used pairs] local pair of each
+    std::vector<int> pair_rep;   // [used pairs] one synapse of each, local to its network
+    std::vector<uint8_t> type2;  // [nt] second-order type
+    std::vector<uint8_t> dup;    // [n_nets] a row has two synapses of one pair
     std::vector<long long> net_syn;
     std::vector<uint8_t> flags;  // NET_HAS2 | NET_PAIR per network
 };
@@ -77,6 +83,8 @@ struct psst_net {
     NetView v{};
     psst::GridView gv{};
     std::vector<psst::ClassLaunch> classes;  // CTA mode: one launch per size class
+    std::vector<std::vector<int>> class_nets;  // the networks of each
+    std::vector<psst::DensePlan> dplans;       // plans of the networks in dense classes
     std::vector<void *> allocs;
     long long step = 0;       // global step index of the current state
     long long rec_reset = 0;  // step at which the record ring was last reset
@@ -478,6 +486,121 @@ int plan_network(const PlanInput &in, int b, const SmemCaps &caps, psst::NetPlan
     return 0;
 }
 
+// ---- dense rows (psst_dense.cu)
+
+struct DenseVariant {
+    int qr, max_block;
+};
+const DenseVariant kDense[] = {
+#define PSST_V(QR, MAXT) {QR, MAXT},
+    PSST_DENSE_VARIANTS(PSST_V)
+#undef PSST_V
+};
+
+// Registers per thread that a block of max_block threads leaves (512 per lane
+// and SM quarter, in units of 8, at most 255).
+int dense_regs(int max_block) {
+    const int r = 512 / ((max_block + 127) / 128) & ~7;
+    return std::min(r, 255);
+}
+
+// The columns of network b: quads per thread, first quad of each type.
+// False when the dense kernel cannot take it.
+bool dense_columns(const PlanInput &in, int b, psst::DensePlan *p) {
+    if (!(in.flags[b] & psst::NET_PAIR) || in.user_K || in.user_block || in.dup[b]) return false;
+    int cnt[PSST_MAX_SYN_TYPES] = {};
+    for (int t = in.pair_off[b]; t < in.pair_off[b + 1]; ++t) ++cnt[in.pair_of[t] % in.nt];
+    std::memset(p, 0, sizeof *p);
+    for (int t = 0; t < in.nt; ++t) {
+        p->tq[t] = p->nq;
+        p->nq += (cnt[t] + 31) / 32;
+    }
+    return p->nq <= 32;
+}
+
+int dense_row_threads(const psst::DensePlan &p, int cl) {
+    int rows = 0;
+    for (int q = 0; q < cl; ++q) rows = std::max(rows, p.split[q + 1] - p.split[q]);
+    return psst::dense_row_threads(rows);
+}
+
+// Largest dynamic shared memory of the network's CTAs.
+long long dense_need(const psst::DensePlan &p, int cl, int qr) {
+    long long need = 0;
+    for (int q = 0; q < cl; ++q) {
+        const psst::DenseLayout y =
+            psst::make_dense_layout(p.split[q + 1] - p.split[q], p.psec[q] - p.psplit[q],
+                                    p.psplit[q + 1] - p.psec[q], p.nq, qr, p.stage_rows);
+        need = std::max<long long>(need, y.bytes);
+    }
+    return need;
+}
+
+// CTAs per SM of a dense class: registers, shared memory.
+int dense_ctas(const SmemCaps &caps, const DenseVariant &d, int threads, long long need) {
+    const int warps = 4 * (512 / dense_regs(d.max_block)), w = threads / 32;
+    return (int)std::min<long long>(warps / w, caps.per_sm / (need + caps.per_cta));
+}
+
+// Rows per CTA, pairs per CTA and variant for network b on a cluster of at
+// least min_cl CTAs (the smallest that fits); 0 if none does.  Of the
+// variants that fit, the one with the most resident warps (up to 16 per SM;
+// `alone`: of this CTA only), then the most quads in registers -- but with 7
+// quads, which leave no registers for the loads of others from shared memory,
+// only when these are all.
+int plan_dense(const PlanInput &in, int b, int min_cl, bool alone, const SmemCaps &caps, psst::DensePlan *p,
+               int *qr) {
+    if (!dense_columns(in, b, p)) return 0;
+    const int n0 = in.net_off[b], N = in.net_off[b + 1] - n0, nt = in.nt;
+    for (int cl = 1; cl <= PSST_MAX_CL; cl *= 2) {
+        if (cl > 1 && N < 2 * cl) break;
+        if (cl < min_cl && N >= 2 * min_cl) continue;
+        int t = in.pair_off[b];
+        for (int q = 0; q <= cl; ++q) {
+            p->split[q] = (int)((long long)q * N / cl);
+            while (t < in.pair_off[b + 1] && in.pair_of[t] / nt < p->split[q]) ++t;
+            p->psplit[q] = t - in.pair_off[b];
+        }
+        for (int q = 0; q < cl; ++q) {
+            p->psec[q] = p->psplit[q];
+            for (int t2 = p->psplit[q]; t2 < p->psplit[q + 1]; ++t2)
+                p->psec[q] += !in.type2[in.pair_of[in.pair_off[b] + t2] % nt];
+        }
+        const int rows = (N + cl - 1) / cl;
+        // up to 48 KB of rows staged at a time while the weights are loaded
+        p->stage_rows = std::max(4, std::min((rows + 3) & ~3, 49152 / (128 * p->nq) & ~3));
+        const int threads = dense_row_threads(*p, cl);
+        int best = 0, best_warps = -1;
+        for (const DenseVariant &d : kDense) {
+            if (threads > d.max_block || d.qr > p->nq || (d.qr == 7 && p->nq > 7)) continue;
+            const long long need = dense_need(*p, cl, d.qr);
+            if (need > caps.max_dyn) continue;
+            const int warps = std::min(16, (alone ? 1 : dense_ctas(caps, d, threads, need)) * threads / 32);
+            if (warps >= best_warps) {
+                best_warps = warps;
+                best = d.qr;
+            }
+        }
+        if (best) {
+            *qr = best;
+            return cl;
+        }
+    }
+    return 0;
+}
+
+// Threads that give every neuron's and every pair's unit one of its own
+// beside the rows'.
+int dense_unit_threads(const psst::DensePlan &p, int cl) {
+    int most = 0;
+    for (int q = 0; q < cl; ++q) {
+        auto w = [](int n) { return (n + 31) & ~31; };
+        most = std::max(most, psst::dense_row_threads(p.split[q + 1] - p.split[q]) + w(p.split[q + 1] - p.split[q]) +
+                                  w(p.psec[q] - p.psplit[q]) + w(p.psplit[q + 1] - p.psec[q]));
+    }
+    return most;
+}
+
 // Per network: do all gates of each (presynaptic neuron, type) pair hold the
 // same value in the state y ([V, m, h, n, r, s], host memory; NULL = rest,
 // all gates 0)?
@@ -616,6 +739,47 @@ int setup_grid(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
     return PSST_OK;
 }
 
+// Columns of the used pairs in the dense kernel's rows: each type's pairs in
+// pair order from the type's first granule.
+cudaError_t upload_columns(psst_net *h, const std::vector<psst::DensePlan> &plans, const std::vector<int> &qr_of) {
+    const PlanInput &in = h->pin;
+    std::vector<unsigned short> col((size_t)h->v.N * in.nt, 0);
+    bool any = false;
+    for (int b = 0; b < in.n_nets; ++b) {
+        if (!qr_of[b]) continue;
+        any = true;
+        int next[PSST_MAX_SYN_TYPES];
+        for (int t = 0; t < in.nt; ++t) next[t] = 32 * plans[b].tq[t];
+        unsigned short *cb = col.data() + (size_t)in.net_off[b] * in.nt;
+        for (int t = in.pair_off[b]; t < in.pair_off[b + 1]; ++t)
+            cb[in.pair_of[t]] = (unsigned short)next[in.pair_of[t] % in.nt]++;
+    }
+    if (!any) return cudaSuccess;
+    // the pairs in the order of their CTAs' units
+    std::vector<int2> pairs(in.pair_of.size());
+    for (int b = 0; b < in.n_nets; ++b) {
+        if (!qr_of[b]) continue;
+        const int p0 = in.pair_off[b];
+        for (int q = 0; q < PSST_MAX_CL && plans[b].psplit[q] < in.pair_off[b + 1] - p0; ++q) {
+            int at[2] = {p0 + plans[b].psplit[q], p0 + plans[b].psec[q]};
+            for (int t = p0 + plans[b].psplit[q]; t < p0 + plans[b].psplit[q + 1]; ++t)
+                pairs[at[in.type2[in.pair_of[t] % in.nt]]++] = make_int2(in.pair_of[t], in.pair_rep[t]);
+        }
+    }
+    if (!h->v.pair_col) {
+        unsigned short *p = nullptr;
+        int2 *dp = nullptr;
+        cudaError_t e = h->alloc(&p, col.size());
+        if (e == cudaSuccess) e = h->alloc(&dp, pairs.size());
+        if (e != cudaSuccess) return e;
+        h->v.pair_col = p;
+        h->v.dense_pair = dp;
+    }
+    cudaError_t e = cudaMemcpy((void *)h->v.dense_pair, pairs.data(), pairs.size() * sizeof(int2), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return e;
+    return cudaMemcpy((void *)h->v.pair_col, col.data(), col.size() * sizeof(col[0]), cudaMemcpyHostToDevice);
+}
+
 // CTA mode: each network's cluster size and work items, size classes by
 // cluster size x CTAs per SM, launch lists (largest networks first).
 int setup_cta(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
@@ -628,6 +792,8 @@ int setup_cta(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
     std::vector<int> cl_of((size_t)n_nets), per_sm((size_t)n_nets);
     std::vector<long long> need((size_t)n_nets);
     std::vector<double> cost((size_t)n_nets);
+    std::vector<psst::DensePlan> dplans((size_t)n_nets);
+    std::vector<int> qr_of((size_t)n_nets, 0);
     std::vector<int> ind_neuron, ind_net;  // neurons of the networks without synapses
     for (int b = 0; b < n_nets; ++b) {
         const int n0 = in.net_off[b], N = in.net_off[b + 1] - n0;
@@ -641,15 +807,55 @@ int setup_cta(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
         }
         if ((long long)N * nt >= 65536)
             return fail(PSST_ERR_UNSUPPORTED, "net %d: %d neurons x %d synapse types must stay below 65536", b, N, nt);
-        const int cl = plan_network(in, b, caps, &plans[b], &need[b]);
+        // what CTA mode accepts is what the item kernel can hold; the dense
+        // kernel then takes the networks that it can (half the item kernel's
+        // time or less per network up to 120 neurons and where SMs are idle,
+        // 0.5 to 0.85 of it above, at 10 to 50% connectivity)
+        int cl = plan_network(in, b, caps, &plans[b], &need[b]);
+        const int dcl = cl ? plan_dense(in, b, in.min_cl, false, caps, &dplans[b], &qr_of[b]) : 0;
+        if (dcl) {
+            cl = dcl;
+            plans[b].K = 0;
+            need[b] = dense_need(dplans[b], dcl, qr_of[b]);
+        }
         if (!cl)
             return fail(PSST_ERR_UNSUPPORTED, "net %d (%d neurons, %lld synapses) does not fit %d CTAs", b, N,
                         in.net_syn[b], PSST_MAX_CL);
         cl_of[b] = cl;
-        per_sm[b] = ctas_per_sm(caps, need[b]);
+        per_sm[b] = dcl ? 0 : ctas_per_sm(caps, need[b]);
         double c = 0;
         for (int i = n0; i < n0 + N; ++i) c += n1[i] + n2[i] + 30.0;
         cost[b] = c;
+    }
+    // SMs left over: networks whose weights do not all fit in registers go to
+    // clusters of twice as many CTAs, the costliest first (240 neurons alone:
+    // 6.7 us per step on one CTA, 4.6 on two, 3.9 on four; results do not
+    // depend on it)
+    int sms = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    if (e != cudaSuccess) return *err = e, cuda_fail(e, "device attributes");
+    long long ctas = 0;
+    for (int b = 0; b < n_nets; ++b) ctas += cl_of[b];
+    if (ctas <= sms)  // every CTA has an SM of its own
+        for (int b = 0; b < n_nets; ++b)
+            if (qr_of[b] && plan_dense(in, b, in.min_cl, true, caps, &dplans[b], &qr_of[b]))
+                need[b] = dense_need(dplans[b], cl_of[b], qr_of[b]);
+    if (in.tune_cl && in.min_cl == 1 && ctas < sms) {
+        std::vector<int> order((size_t)n_nets);
+        std::iota(order.begin(), order.end(), 0);
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b2) { return cost[a] > cost[b2]; });
+        for (int mc = 2; mc <= PSST_MAX_CL; mc *= 2)
+            for (int b : order) {
+                if (cl_of[b] != mc / 2 || qr_of[b] == 0 || qr_of[b] >= dplans[b].nq || ctas + mc / 2 > sms) continue;
+                psst::DensePlan p;
+                int qr = 0;
+                if (plan_dense(in, b, mc, true, caps, &p, &qr) != mc) continue;
+                dplans[b] = p;
+                qr_of[b] = qr;
+                cl_of[b] = mc;
+                need[b] = dense_need(p, mc, qr);
+                ctas += mc / 2;
+            }
     }
     std::vector<int> all_lists;
     std::vector<std::pair<int, int>> ranges;
@@ -657,7 +863,7 @@ int setup_cta(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
         for (int k = 1; k <= 4; ++k) {
             std::vector<int> list;
             for (int b = 0; b < n_nets; ++b)
-                if (cl_of[b] == cl && per_sm[b] == k) list.push_back(b);
+                if (!qr_of[b] && cl_of[b] == cl && per_sm[b] == k) list.push_back(b);
             if (list.empty()) continue;
             std::stable_sort(list.begin(), list.end(), [&](int a, int b2) { return cost[a] > cost[b2]; });
             psst::ClassLaunch c{};
@@ -675,19 +881,66 @@ int setup_cta(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
             h->classes.push_back(c);
         }
     }
+    // dense classes: by cluster size, block (rounded up to 64 threads) and variant
+    {
+        std::map<std::tuple<int, int, int>, std::vector<int>> groups;
+        for (int b = 0; b < n_nets; ++b)
+            if (qr_of[b])
+                groups[{-cl_of[b], -((dense_row_threads(dplans[b], cl_of[b]) + 63) / 64), qr_of[b]}]
+                    .push_back(b);
+        for (auto &kv : groups) {
+            std::vector<int> &list = kv.second;
+            std::stable_sort(list.begin(), list.end(), [&](int a, int b2) { return cost[a] > cost[b2]; });
+            psst::ClassLaunch c{};
+            c.cl = -std::get<0>(kv.first);
+            c.qr = std::get<2>(kv.first);
+            c.n_nets = (int)list.size();
+            for (int b : list) {
+                c.smem = (int)std::max<long long>(c.smem, need[b]);
+                c.rows = std::max(c.rows, dense_row_threads(dplans[b], c.cl));
+            }
+            // threads of their own for the neurons' and pairs' units, as far
+            // as they take no CTA's place on its SM (150 neurons, two networks
+            // per SM: 7.7 -> 7.5 us per step; 20 neurons 2.2 -> 1.9; 90 neurons
+            // at the price of the second CTA: 3.2 -> 5.8)
+            int units = 0;
+            for (int b : list) units = std::max(units, dense_unit_threads(dplans[b], c.cl));
+            const DenseVariant &d = *std::find_if(std::begin(kDense), std::end(kDense),
+                                                  [&](const DenseVariant &x) { return x.qr == c.qr; });
+            const int keep = (int)std::min<long long>(dense_ctas(caps, d, c.rows, c.smem), (ctas + sms - 1) / sms);
+            c.block = c.rows;
+            while (c.block + 32 <= std::min(units, d.max_block) && dense_ctas(caps, d, c.block + 32, c.smem) >= keep)
+                c.block += 32;
+            ranges.push_back({(int)all_lists.size(), (int)list.size()});
+            all_lists.insert(all_lists.end(), list.begin(), list.end());
+            h->classes.push_back(c);
+        }
+    }
     int *dl = nullptr;
     psst::NetPlan *dp = nullptr;
-    cudaError_t e = upload(h, &dl, all_lists.data(), all_lists.size());
+    psst::DensePlan *ddp = nullptr;
+    e = upload(h, &dl, all_lists.data(), all_lists.size());
     if (e == cudaSuccess) e = upload(h, &dp, plans.data(), plans.size());
+    if (e == cudaSuccess) e = upload(h, &ddp, dplans.data(), dplans.size());
+    if (e == cudaSuccess) e = upload_columns(h, dplans, qr_of);
     for (size_t i = 0; e == cudaSuccess && i < h->classes.size(); ++i) {
         h->classes[i].list = dl + ranges[i].first;
         h->classes[i].plans = dp;
-        e = psst::cta_prepare(h->classes[i].cl, caps.max_dyn);
+        h->classes[i].dplans = ddp;
+        if (h->classes[i].qr) {
+            e = psst::dense_prepare(h->classes[i].qr, caps.max_dyn);
+        } else {
+            e = psst::cta_prepare(h->classes[i].cl, caps.max_dyn);
+        }
     }
     if (e == cudaSuccess && !ind_neuron.empty() && !h->d_ind_neuron) {
         e = upload(h, &h->d_ind_neuron, ind_neuron.data(), ind_neuron.size());
         if (e == cudaSuccess) e = upload(h, &h->d_ind_net, ind_net.data(), ind_net.size());
     }
+    h->class_nets.clear();
+    for (const auto &r : ranges)
+        h->class_nets.emplace_back(all_lists.begin() + r.first, all_lists.begin() + r.first + r.second);
+    h->dplans = dplans;
     h->n_ind_neurons = (int)ind_neuron.size();
     h->n_ind_nets = 0;
     for (int b = 0; b < n_nets; ++b) h->n_ind_nets += in.net_syn[b] == 0;
@@ -766,18 +1019,30 @@ int psst_create_network(const psst_network_desc *d, const psst_allocator *a, pss
                            (uni[b] && !pin.force_synapse_gates ? psst::NET_PAIR : 0);
     }
     // compact index of each network's used (presynaptic neuron, type) pairs
-    std::vector<int> ptix((size_t)N * nt, -1), pof;
-    std::vector<int> &pair_off = pin.pair_off;
+    std::vector<int> ptix((size_t)N * nt, -1);
+    std::vector<int> &pair_off = pin.pair_off, &pof = pin.pair_of;
+    for (int t = 0; t < nt; ++t) pin.type2.push_back(d->syn_params[(size_t)t * PSST_SYN_NPARAM] != 0.0f);
     pair_off.assign((size_t)n_nets + 1, 0);
+    pin.dup.assign((size_t)n_nets, 0);
     for (int b = 0; b < n_nets; ++b) {
         const long long n0 = d->net_neuron_off[b], nb = d->net_neuron_off[b + 1] - n0;
         int *tb = ptix.data() + n0 * nt;
-        for (long long k = d->row_ptr[n0]; k < d->row_ptr[n0 + nb]; ++k) tb[(size_t)d->pre[k] * nt + d->syn_type[k]] = 0;
+        // mark each pair with the last row that used it (row + 1, local), and
+        // keep one of its synapses: the last
+        std::vector<int> last_syn((size_t)nb * nt);
+        for (long long i = n0; i < n0 + nb; ++i)
+            for (long long k = d->row_ptr[i]; k < d->row_ptr[i + 1]; ++k) {
+                const size_t p = (size_t)d->pre[k] * nt + d->syn_type[k];
+                if (tb[p] == (int)(i - n0)) pin.dup[b] = 1;
+                tb[p] = (int)(i - n0);
+                last_syn[p] = (int)(k - d->row_ptr[n0]);
+            }
         pair_off[b] = (int)pof.size();
         for (long long p = 0; p < nb * nt; ++p)
-            if (tb[p] == 0) {
+            if (tb[p] >= 0) {
                 tb[p] = (int)pof.size() - pair_off[b];
                 pof.push_back((int)p);
+                pin.pair_rep.push_back(last_syn[p]);
             }
     }
     pair_off[n_nets] = (int)pof.size();
@@ -927,6 +1192,10 @@ namespace {
 
 int launch_chunks(psst_net *h, long long step0, long long n_steps, long long chunk, cudaStream_t st);
 
+cudaError_t class_launch(const NetView &v, const psst::ClassLaunch &c, long long step0, int n, cudaStream_t st) {
+    return c.qr ? psst::dense_launch(v, c, step0, n, st) : psst::cta_launch(v, c, step0, n, st);
+}
+
 // Launch the kernels for n_steps steps starting at global step `step0`.
 int launch_steps(psst_net *h, long long step0, long long n_steps, cudaStream_t st) {
     const long long chunk = 1LL << 30;
@@ -962,7 +1231,7 @@ int launch_chunks(psst_net *h, long long step0, long long n_steps, long long chu
         } else {
             const bool fork = !h->class_streams.empty();
             for (size_t c = 0; c < h->classes.size(); ++c) {
-                cudaError_t e = psst::cta_launch(h->v, h->classes[c], step0 + done, n,
+                cudaError_t e = class_launch(h->v, h->classes[c], step0 + done, n,
                                                  fork ? h->class_streams[c] : st);
                 if (e != cudaSuccess) return cuda_fail(e, "psst_integrate launch");
                 ++h->launches;
@@ -1147,37 +1416,66 @@ int psst_autotune(psst_net *h, int64_t trial_steps, void *stream) {
         // default CTA keeps 1024 threads per SM (64 registers each); the
         // trials try twice, once, half and a quarter of that size, each with
         // the planned copies of the per-pair gate table and with one copy
-        const int base = c.block;
+        std::vector<psst::ClassLaunch> trials;
+        if (c.qr) {
+            // per register budget the most quads that fit, unless the default
+            // has more than twice as many; each with just the rows' threads,
+            // 128 more and the default's
+            int last_block = 0;
+            for (int k = (int)std::size(kDense) - 1; k >= 0; --k) {
+                const DenseVariant &d = kDense[k];
+                if (d.max_block == last_block || 2 * d.qr < c.qr || c.rows > d.max_block) continue;
+                psst::ClassLaunch t = c;
+                t.qr = d.qr;
+                long long need = 0;
+                bool fits = true;
+                for (int b : h->class_nets[ci]) {
+                    fits = fits && d.qr <= h->dplans[b].nq;
+                    if (fits) need = std::max(need, dense_need(h->dplans[b], c.cl, d.qr));
+                }
+                if (!fits || need > h->caps.max_dyn || psst::dense_prepare(d.qr, h->caps.max_dyn) != cudaSuccess)
+                    continue;
+                last_block = d.max_block;
+                t.smem = (int)need;
+                int tried[3] = {0, 0, 0};
+                for (int q = 0; q < 3; ++q) {
+                    t.block = std::min(d.max_block, q == 0 ? c.rows : q == 1 ? c.rows + 128 : std::max(c.rows, c.block));
+                    tried[q] = t.block;
+                    if ((q > 0 && t.block == tried[0]) || (q > 1 && t.block == tried[1])) continue;
+                    trials.push_back(t);
+                }
+            }
+        } else {
+            for (int trial = 0; trial < 8; ++trial) {
+                psst::ClassLaunch t = c;
+                t.block = trial / 2 == 0 ? 2 * c.block : c.block >> (trial / 2 - 1);
+                t.lrep_cap = trial % 2 ? 0 : c.lrep_cap;
+                if (t.block > 1024 || t.block < 64 || t.block % 32 || (trial % 2 && c.lrep_cap == 0)) continue;
+                trials.push_back(t);
+            }
+        }
         float best = 1e30f;
-        int best_block = base, best_cap = c.lrep_cap;
-        for (int trial = 0; trial < 8; ++trial) {
-            const int b = trial / 2 == 0 ? 2 * base : base >> (trial / 2 - 1);
-            const int cap = trial % 2 ? 0 : c.lrep_cap;
-            if (b > 1024 || b < 64 || b % 32 || (trial % 2 && c.lrep_cap == 0)) continue;
-            psst::ClassLaunch t = c;
-            t.block = b;
-            t.lrep_cap = cap;
-            const int n = (int)std::min<long long>(trial_steps, 1 << 20);
-            e = psst::cta_launch(h->v, t, 0, n, st);  // warm-up
+        psst::ClassLaunch pick = c;
+        const int n = (int)std::min<long long>(trial_steps, 1 << 20);
+        for (const psst::ClassLaunch &t : trials) {
+            e = class_launch(h->v, t, 0, n, st);  // warm-up
             if (e != cudaSuccess) {
                 cudaGetLastError();  // a shape that cannot launch is skipped
                 e = cudaSuccess;
                 continue;
             }
             cudaEventRecord(ev0, st);
-            e = psst::cta_launch(h->v, t, 0, n, st);
+            e = class_launch(h->v, t, 0, n, st);
             cudaEventRecord(ev1, st);
             if (e == cudaSuccess) e = cudaEventSynchronize(ev1);
             float ms = 0.0f;
             if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev0, ev1);
             if (e == cudaSuccess && ms < best) {
                 best = ms;
-                best_block = b;
-                best_cap = cap;
+                pick = t;
             }
         }
-        c.block = best_block;
-        c.lrep_cap = best_cap;
+        c = pick;
     }
     h->v.rec_stride = stride;
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->v.state, h->tune_buf, dim * sizeof(float), cudaMemcpyDeviceToDevice, st);

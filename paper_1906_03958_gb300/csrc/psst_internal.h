@@ -15,7 +15,22 @@ struct ClassLaunch {
     const int *list;      // [n_nets] device: network indices, largest first
     const NetPlan *plans; // [all nets] device
     int lrep_cap;         // per-pair gates: at most 2^lrep_cap copies of the gate table (autotuned)
+    int qr;               // dense kernel: quads per thread in registers (0: the item kernel)
+    int rows;             // dense kernel: threads that hold rows (the smallest block)
+    const DensePlan *dplans; // dense kernel: [all nets] device
 };
+
+// Dense kernel (psst_dense.cu): quads per thread held in registers and the
+// largest block of each compiled variant.  An SM quarter holds 512 registers
+// per lane, so the block sizes with 6, 5, 4, 3 and 2 warps a quarter leave
+// 80, 96, 128, 168 and 255 registers a thread: 16 per quad and about 55 for
+// everything else.  A quad in shared memory costs four 16-byte loads more and
+// shows: a network of 300 neurons on 4 CTAs takes 4.1 us per step with all 10
+// quads in registers, 5.6 with 2 (240 neurons on 2: 4.6 with 6 of 8, 5.6 with 1).
+#define PSST_DENSE_VARIANTS(X) \
+    X(1, 768) X(2, 640) X(3, 512) X(4, 512) X(5, 384) X(6, 384) X(7, 384) X(8, 256) X(9, 256) X(10, 256)
+cudaError_t dense_prepare(int qr, int max_smem);
+cudaError_t dense_launch(const NetView &v, const ClassLaunch &c, long long step0, int nsteps, cudaStream_t stream);
 
 // CTA/cluster batched kernel (psst_cta.cu).
 int cta_static_smem();

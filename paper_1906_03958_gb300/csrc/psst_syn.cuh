@@ -615,26 +615,42 @@ struct VPre {
     float acc;   // RK4 sum of V's stage slopes so far
 };
 
+// Parameters of one neuron (invC: 1 / C).
+struct NeuronPrm {
+    float invC, gNa, gK, gL, ENa, EK, EL, gKL, EKL;
+};
+
+__device__ __forceinline__ NeuronPrm load_neuron_prm(const NetView &v, long long gi) {
+    const float *p = v.nparams + (long long)v.neuron_type[gi] * PSST_NEURON_NPARAM;
+    return NeuronPrm{1.0f / p[NP_C], p[NP_GNA], p[NP_GK], p[NP_GL], p[NP_ENA], p[NP_EK], p[NP_EL], p[NP_GKL], p[NP_EKL]};
+}
+
+// I_ext - I_ion: explicit roundings (no contraction left to the compiler),
+// so that every kernel evaluates the same operations in whatever context it
+// is inlined.
+__device__ __forceinline__ float ionic_rest(const NeuronPrm &P, float V, float m, float h, float nn, float iext) {
+    const float m3h = __fmul_rn(__fmul_rn(__fmul_rn(m, m), m), h);
+    const float n2 = __fmul_rn(nn, nn), n4 = __fmul_rn(n2, n2);
+    float iion = __fmul_rn(__fmul_rn(P.gNa, m3h), __fsub_rn(V, P.ENa));
+    iion = fmaf(__fmul_rn(P.gK, n4), __fsub_rn(V, P.EK), iion);
+    iion = fmaf(P.gL, __fsub_rn(V, P.EL), iion);
+    iion = fmaf(P.gKL, __fsub_rn(V, P.EKL), iion);
+    return __fsub_rn(iext, iion);
+}
+
 template <class SG>
 __device__ __forceinline__ VPre neuron_v_pre(const SG &sg, int i, int n, float V, const float *ysc,
                                              const float *y0, const float *ylo, const float *acc, const float *prm,
                                              float iext) {
-    const bool FIRST = sg.first;
-    const float m = ysc[i], h = ysc[n + i], nn = ysc[2 * n + i];
-    // explicit roundings (no contraction left to the compiler), so that every
-    // kernel evaluates the same operations in whatever context it is inlined
-    const float m3h = __fmul_rn(__fmul_rn(__fmul_rn(m, m), m), h);
-    const float n2 = __fmul_rn(nn, nn), n4 = __fmul_rn(n2, n2);
-    float iion = __fmul_rn(__fmul_rn(prm[NP_GNA * n + i], m3h), __fsub_rn(V, prm[NP_ENA * n + i]));
-    iion = fmaf(__fmul_rn(prm[NP_GK * n + i], n4), __fsub_rn(V, prm[NP_EK * n + i]), iion);
-    iion = fmaf(prm[NP_GL * n + i], __fsub_rn(V, prm[NP_EL * n + i]), iion);
-    iion = fmaf(prm[NP_GKL * n + i], __fsub_rn(V, prm[NP_EKL * n + i]), iion);
+    const NeuronPrm P{prm[NP_C * n + i],  prm[NP_GNA * n + i], prm[NP_GK * n + i],
+                      prm[NP_GL * n + i], prm[NP_ENA * n + i], prm[NP_EK * n + i],
+                      prm[NP_EL * n + i], prm[NP_GKL * n + i], prm[NP_EKL * n + i]};
     VPre r;
-    r.ie = __fsub_rn(iext, iion);
-    r.invC = prm[NP_C * n + i];  // prm row 0 holds 1/C
+    r.ie = ionic_rest(P, V, ysc[i], ysc[n + i], ysc[2 * n + i], iext);
+    r.invC = P.invC;
     r.y0 = y0[i];
     r.lo = ylo[i];
-    r.acc = FIRST ? 0.0f : acc[i];
+    r.acc = sg.first ? 0.0f : acc[i];
     return r;
 }
 
