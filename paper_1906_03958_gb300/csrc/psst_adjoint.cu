@@ -870,7 +870,11 @@ cudaError_t adj_launch(const NetView &v, const AdjView &av, long long step0, int
     cfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg, kern, v, av, step0, nsteps);
     if (e != cudaSuccess) return e;
-    adj_reduce_types<<<n_types, 32, 0, stream>>>(v.neuron_type, v.N, av.gp_neuron, n_types, grad_np);
+    return adj_reduce(v, av.gp_neuron, n_types, grad_np, stream);
+}
+
+cudaError_t adj_reduce(const NetView &v, const double *gp_neuron, int n_types, float *grad_np, cudaStream_t stream) {
+    adj_reduce_types<<<n_types, 32, 0, stream>>>(v.neuron_type, v.N, gp_neuron, n_types, grad_np);
     return cudaGetLastError();
 }
 

@@ -107,6 +107,14 @@ struct psst_net {
     double *adj_gtot = nullptr;
     double *adj_gpn = nullptr;
     long long adj_seg_cap = 0;
+    // adjoint over dense rows: 0 not planned yet, 1 planned, -1 not for these networks
+    int adjd_state = 0, adjd_Q = 0, adjd_threads = 0, adjd_smem = 0;
+    long long adjd_span = -1;  // steps of a segment buffer the uploaded plans are laid out for
+    std::vector<psst::AdjDensePlan> adjd_plans;
+    psst::AdjDensePlan *d_adjd_plans = nullptr;
+    int4 *d_adjd_pair = nullptr;
+    unsigned short *d_adjd_slot = nullptr, *d_adjd_col = nullptr;
+    float2 *adjd_gtot = nullptr;
     int adj_ckpt_every = 0;
     // checkpoints recorded by psst_integrate for a later psst_adjoint
     int rec_ck_every = 0;
@@ -1688,6 +1696,126 @@ int psst_set_neuron_params(psst_net *h, const float *p, size_t n, int on_device,
     return e == cudaSuccess ? PSST_OK : cuda_fail(e, "psst_set_neuron_params");
 }
 
+// Plan of the adjoint over dense rows (psst_adjdense.cu): for handles whose
+// networks all have at most 128 neurons, 4 synapse types, 160 slots of used
+// pairs and no two synapses of one pair in a row.
+static int plan_adj_dense(psst_net *h) {
+    const PlanInput &in = h->pin;
+    const int n_nets = in.n_nets, nt = in.nt;
+    const int ns = h->v.method == PSST_METHOD_EULER ? 1 : h->v.method == PSST_METHOD_TABLEAU ? h->v.rk_ns : 4;
+    h->adjd_state = -1;
+    if (nt > psst::ADJ_DENSE_TYPES) return PSST_OK;
+    int Q = 1;
+    for (int b = 0; b < n_nets; ++b) {
+        const int N = in.net_off[b + 1] - in.net_off[b];
+        if (in.dup[b] || N < 1 || N > 32 * psst::ADJ_DENSE_Q) return PSST_OK;
+        Q = std::max(Q, (N + 31) / 32);
+    }
+    std::vector<psst::AdjDensePlan> plans((size_t)n_nets);
+    std::vector<int4> pair(in.pair_of.size());
+    std::vector<unsigned short> slot((size_t)h->v.N * nt, 0), col((size_t)h->v.N * nt, 0);
+    int threads = 0;
+    long long need = 0, grad = 0;
+    for (int b = 0; b < n_nets; ++b) {
+        psst::AdjDensePlan &p = plans[b];
+        std::memset(&p, 0, sizeof p);
+        const int n0 = in.net_off[b], N = in.net_off[b + 1] - n0, p0 = in.pair_off[b], np = in.pair_off[b + 1] - p0;
+        int cnt[PSST_MAX_SYN_TYPES] = {}, seen[PSST_MAX_SYN_TYPES] = {};
+        for (int t = 0; t < np; ++t) ++cnt[in.pair_of[p0 + t] % nt];
+        for (int t = 0; t < nt; ++t) {
+            p.tq[t] = p.nq;
+            p.nq += (cnt[t] + 31) / 32;
+            p.ts[t] = p.Mp;
+            p.Mp += (cnt[t] + 3) & ~3;
+            (in.type2[t] ? p.np2 : p.np1) += cnt[t];
+        }
+        p.Mp = std::max(16, (p.Mp + 15) & ~15);
+        p.nq = std::max(p.nq, Q + 1);
+        if (2 * p.Mp + psst::ADJ_DENSE_NEURONS > psst::ADJ_DENSE_THREADS) return PSST_OK;
+        p.pair0 = p0;
+        int at[2] = {p0, p0 + p.np1};
+        for (int t = 0; t < np; ++t) {
+            const int ci = in.pair_of[p0 + t], ty = ci % nt, k = seen[ty]++;
+            slot[(size_t)n0 * nt + ci] = (unsigned short)(p.ts[ty] + k);
+            col[(size_t)n0 * nt + ci] = (unsigned short)(32 * p.tq[ty] + k);
+            pair[at[in.type2[ty]]++] = make_int4(ci, in.pair_rep[p0 + t], p.ts[ty] + k, 32 * p.tq[ty] + k);
+        }
+        const long long rec = 2LL * 4 * ns * psst::adj_stage_floats(N, p.Mp);
+        p.rows = std::max(4, std::min((N + 3) & ~3, 49152 / (128 * p.nq) & ~3));
+        p.slots = std::min<int>(p.Mp, (int)(std::max(rec, 65536LL) / (128 * Q)) & ~3);
+        p.grad_off = grad;
+        grad += 8LL * Q * 2 * p.Mp;
+        need = std::max<long long>(need, psst::make_adj_layout(N, nt, p.Mp, np, p.np2, p.nq, Q + 1, Q, ns, p.rows,
+                                                               p.slots).bytes);
+        threads = std::max({threads, psst::dense_row_threads(N), 2 * p.Mp + psst::ADJ_DENSE_NEURONS});
+    }
+    if (need > h->max_dyn) return PSST_OK;
+    cudaError_t e = h->alloc(&h->d_adjd_plans, plans.size());
+    if (e == cudaSuccess) e = upload(h, &h->d_adjd_pair, pair.data(), pair.size());
+    if (e == cudaSuccess) e = upload(h, &h->d_adjd_slot, slot.data(), slot.size());
+    if (e == cudaSuccess) e = upload(h, &h->d_adjd_col, col.data(), col.size());
+    if (e == cudaSuccess) e = h->alloc(&h->adjd_gtot, (size_t)grad * 2);
+    if (e == cudaSuccess && !h->adj_gpn) e = h->alloc(&h->adj_gpn, (size_t)h->v.N * 9);
+    if (e == cudaSuccess && !h->adj_gy0) e = h->alloc(&h->adj_gy0, (size_t)h->v.N * 4);
+    if (e != cudaSuccess) {
+        h->adjd_state = 0;
+        return cuda_fail(e, "psst_adjoint buffers");
+    }
+    h->adjd_plans = plans;
+    h->adjd_Q = Q;
+    h->adjd_threads = threads;
+    h->adjd_smem = (int)need;
+    h->adjd_span = -1;
+    h->adjd_state = 1;
+    return PSST_OK;
+}
+
+// The adjoint over dense rows of the recorded span.
+static int adjoint_dense(psst_net *h, long long s0, int n_steps, int ckpt_every, const float *dL_dV, int n_frames,
+                         float *grad_w, float *grad_np, float *grad_state0, cudaStream_t st) {
+    const int ns = h->v.method == PSST_METHOD_EULER ? 1 : h->v.method == PSST_METHOD_TABLEAU ? h->v.rk_ns : 4;
+    const long long span = std::min(ckpt_every, n_steps);
+    if (h->adjd_span != span) {
+        long long total = 0;
+        for (int b = 0; b < h->pin.n_nets; ++b) {
+            psst::AdjDensePlan &p = h->adjd_plans[b];
+            p.seg_off = total;
+            total += 2 * span * ns * psst::adj_stage_floats(h->pin.net_off[b + 1] - h->pin.net_off[b], p.Mp);
+        }
+        cudaError_t e = cudaSuccess;
+        if (total > h->adj_seg_cap) {
+            e = h->alloc(&h->adj_seg, (size_t)total);
+            h->adj_seg_cap = e == cudaSuccess ? total : 0;
+        }
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(h->d_adjd_plans, h->adjd_plans.data(), h->adjd_plans.size() * sizeof(psst::AdjDensePlan),
+                                cudaMemcpyHostToDevice, st);
+        if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint storage");
+        h->adjd_span = span;
+    }
+    psst::AdjDenseView av{};
+    av.plan = h->d_adjd_plans;
+    av.pair = h->d_adjd_pair;
+    av.slot = h->d_adjd_slot;
+    av.col = h->d_adjd_col;
+    av.ckpt_every = ckpt_every;
+    av.ck = h->rec_ck;
+    av.ck_lo = h->rec_ck_lo;
+    av.dim = 4 * h->v.N + 2 * h->v.S;
+    av.seg = h->adj_seg;
+    av.gtot = h->adjd_gtot;
+    av.dLdV = dL_dV;
+    av.n_frames = n_frames;
+    av.grad_w = grad_w;
+    av.gp_neuron = h->adj_gpn;
+    av.grad_y0 = grad_state0 ? grad_state0 : h->adj_gy0;
+    const cudaError_t e = psst::adj_dense_launch(h->v, av, h->adjd_Q, h->adjd_threads, h->adjd_smem, s0, n_steps,
+                                                 h->n_ntypes, grad_np, st);
+    if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint launch");
+    h->launches = 2;
+    return PSST_OK;
+}
+
 int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_frames, int32_t ckpt_every,
                  float *grad_w, float *grad_neuron_params, float *grad_state0, void *stream) {
     if (!h || !grad_w || !grad_neuron_params) return fail(PSST_ERR_INVALID_ARG, "NULL argument");
@@ -1737,6 +1865,16 @@ int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_fra
         if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint state copy");
     }
     ckpt_every = h->rec_ck_spacing;
+    // small networks with one gate per pair: the adjoint over dense rows
+    bool pairs = true;
+    for (uint8_t f : h->pin.flags) pairs = pairs && (f & psst::NET_PAIR);
+    if (pairs && h->adjd_state == 0) {
+        const int rc = plan_adj_dense(h);
+        if (rc) return rc;
+    }
+    if (pairs && h->adjd_state == 1)
+        return adjoint_dense(h, s0, (int)n_steps, ckpt_every, dL_dV, (int)n_frames, grad_w, grad_neuron_params,
+                             grad_state0, (cudaStream_t)stream);
     // per-network plan (host copy of the CSR offsets is not kept: read them back once)
     if (h->adj_K.empty()) {
         std::vector<int> off((size_t)n_nets + 1);
@@ -1825,8 +1963,8 @@ int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_fra
         if (e == cudaSuccess) e = upload(h, &h->d_cslotoff, cslot_off.data(), cslot_off.size());
         if (e == cudaSuccess) e = h->alloc(&h->adj_gpart, (size_t)slots / 4);
         if (e == cudaSuccess) e = h->alloc(&h->adj_gtot, (size_t)slots);
-        if (e == cudaSuccess) e = h->alloc(&h->adj_gpn, (size_t)h->v.N * 9);
-        if (e == cudaSuccess) e = h->alloc(&h->adj_gy0, (size_t)h->v.N * 4);
+        if (e == cudaSuccess && !h->adj_gpn) e = h->alloc(&h->adj_gpn, (size_t)h->v.N * 9);
+        if (e == cudaSuccess && !h->adj_gy0) e = h->alloc(&h->adj_gy0, (size_t)h->v.N * 4);
         if (e == cudaSuccess) e = h->alloc(&h->d_segoff, (size_t)n_nets);
         if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint buffers");
     }
@@ -1843,6 +1981,7 @@ int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_fra
             sg[b] = seg_total;
             seg_total += 2LL * std::min<long long>(ckpt_every, n_steps) * step_floats;  // two buffers
         }
+        h->adjd_span = -1;  // the buffer's layout is this path's now
         if (seg_total > h->adj_seg_cap) {
             e = h->alloc(&h->adj_seg, (size_t)seg_total);
             h->adj_seg_cap = seg_total;

@@ -41,6 +41,7 @@
 
 #include <type_traits>
 
+#include "psst_dense.cuh"
 #include "psst_device.cuh"
 #include "psst_internal.h"
 #include "psst_syn.cuh"
@@ -48,12 +49,6 @@
 namespace psst {
 
 namespace {
-
-extern __shared__ __align__(16) unsigned char dsm[];
-
-// Shared memory at byte offset o.
-__device__ __forceinline__ float &F1(int o) { return *(float *)(dsm + o); }
-__device__ __forceinline__ float4 &F4(int o) { return *(float4 *)(dsm + o); }
 
 __device__ __forceinline__ unsigned cluster_rank() {
     unsigned r;
@@ -76,106 +71,6 @@ __device__ __forceinline__ void put(int o, int cl, float x) {
         asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(raddr) : "r"(laddr), "r"(q));
         asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(raddr), "f"(x) : "memory");
     }
-}
-
-// One gate variable with rates al, be: st (step-start value, its remainder,
-// the step's running sum, stage value) advanced by one stage, the step's last
-// if LAST, with the operations of neuron_gates (psst_syn.cuh).  Running sums
-// start a step at 0 here and everywhere below: the first stage's term w d is
-// fma(w, d, 0).
-template <bool LAST>
-__device__ __forceinline__ void gate_update(const StageCoef &c, float al, float be, float4 &st) {
-    const float d = fmaf(al, __fsub_rn(1.0f, st.w), -__fmul_rn(be, st.w));
-    const float ac = fmaf(c.w, d, st.z);
-    if (!LAST) {
-        st.z = ac;
-        st.w = ext_stage(st.x, st.y, c.cn, d);
-    } else {
-        ext_step(st.x, st.y, c.fin, ac);
-        st.z = 0.0f;
-        st.w = st.x;
-    }
-}
-
-// One pair's r at its neuron's potential V, sp its type's table row: st
-// (step-start gate, remainder, stage map P, Qm), acc the step's running sums,
-// with the operations of coef_update, pair_step and pair_gate; returns the
-// next stage's r.
-template <bool LAST>
-__device__ __forceinline__ float pair_unit(const StageCoef &c, const float *sp, float V, float4 &st, float2 &acc) {
-    const float a_ = __fmul_rn(sp[SP_A], transmitter(V, sp)), bb = __fadd_rn(a_, sp[SP_B]);
-    const float kP = fmaf(-bb, st.z, a_), kQ = fmaf(-bb, st.w, -bb);
-    const float aP = fmaf(c.w, kP, acc.x);
-    const float aQ = fmaf(c.w, kQ, acc.y);
-    if (!LAST) {
-        acc = make_float2(aP, aQ);
-        st.z = __fmul_rn(c.cn, kP);
-        st.w = __fmul_rn(c.cn, kQ);
-        return __fadd_rn(st.x, __fadd_rn(fmaf(st.w, st.x, st.z), st.y));
-    }
-    ext_add(st.x, st.y, fmaf(__fmul_rn(c.fin, aQ), st.x, __fmul_rn(c.fin, aP)));
-    st.z = st.w = 0.0f;
-    acc = make_float2(0.0f, 0.0f);
-    return __fadd_rn(st.x, st.y);
-}
-
-__device__ __forceinline__ float second_gate(float s, float Kd) {
-    const float s2 = __fmul_rn(s, s), s4 = __fmul_rn(s2, s2);
-    return __fdiv_rn(s4, __fadd_rn(s4, Kd));
-}
-
-// The second gate of a second-order pair (r0 its step-start r, P and Qm this
-// stage's map of r): q (step-start s, remainder, stage map U, X), z (map Zm,
-// running sums); returns the next stage's G = s^4 / (s^4 + Kd).
-template <bool LAST>
-__device__ __forceinline__ float pair_unit2(const StageCoef &c, const float *sp, float r0, float P, float Qm, float4 &q,
-                                            float4 &z) {
-    const float K3 = sp[SP_K3], K4 = sp[SP_K4];
-    const float kU = fmaf(K3, P, __fmul_rn(-K4, q.z)), kX = fmaf(K3, Qm, fmaf(-K4, q.w, K3));
-    const float kZ = fmaf(-K4, z.x, -K4);
-    const float aU = fmaf(c.w, kU, z.y);
-    const float aX = fmaf(c.w, kX, z.z);
-    const float aZ = fmaf(c.w, kZ, z.w);
-    float s;
-    if (!LAST) {
-        z = make_float4(__fmul_rn(c.cn, kZ), aU, aX, aZ);
-        q.z = __fmul_rn(c.cn, kU);
-        q.w = __fmul_rn(c.cn, kX);
-        s = __fadd_rn(q.x, __fadd_rn(fmaf(z.x, q.x, fmaf(q.w, r0, q.z)), q.y));
-    } else {
-        ext_add(q.x, q.y, fmaf(__fmul_rn(c.fin, aZ), q.x,
-                               fmaf(__fmul_rn(c.fin, aX), r0, __fmul_rn(c.fin, aU))));
-        q.z = q.w = 0.0f;
-        z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        s = __fadd_rn(q.x, q.y);
-    }
-    return second_gate(s, sp[SP_KD]);
-}
-
-// Four rows' currents over one quad of columns with reversal potential E.
-__device__ __forceinline__ void quad(const float4 (&w)[4], float4 g, float E, const float4 &V, float (&I)[4]) {
-    const float Vr[4] = {V.x, V.y, V.z, V.w};
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        float a = __fmul_rn(w[r].x, g.x);
-        a = fmaf(w[r].y, g.y, a);
-        a = fmaf(w[r].z, g.z, a);
-        a = fmaf(w[r].w, g.w, a);
-        I[r] = fmaf(a, __fsub_rn(Vr[r], E), I[r]);
-    }
-}
-
-// Sum over the eight threads of a row group: thread l gets row
-// 2 (l & 1) + (l >> 1 & 1).
-__device__ __forceinline__ float row_sum(const float (&a)[4], int l) {
-    const bool b0 = l & 1, b1 = l & 2;
-    float x0 = __shfl_xor_sync(0xffffffffu, b0 ? a[0] : a[2], 1);
-    float x1 = __shfl_xor_sync(0xffffffffu, b0 ? a[1] : a[3], 1);
-    x0 = __fadd_rn(b0 ? a[2] : a[0], x0);
-    x1 = __fadd_rn(b0 ? a[3] : a[1], x1);
-    const float y = __shfl_xor_sync(0xffffffffu, b1 ? x0 : x1, 2);
-    x0 = __fadd_rn(b1 ? x1 : x0, y);
-    return __fadd_rn(x0, __shfl_xor_sync(0xffffffffu, x0, 4));
 }
 
 template <int QR>

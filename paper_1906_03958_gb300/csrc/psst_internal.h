@@ -55,4 +55,15 @@ long long adj_segment_floats(int method, int rk_ns, int N, int nt);
 cudaError_t adj_launch(const NetView &v, const AdjView &av, long long step0, int nsteps, int smem, int n_types,
                        float *grad_np, cudaStream_t stream);
 
+
+// The adjoint over dense rows (psst_adjdense.cu): networks of at most
+// 32 x ADJ_DENSE_Q neurons and ADJ_DENSE_TYPES synapse types whose pair slots
+// (two threads each) leave ADJ_DENSE_NEURONS of the threads to the neurons; Q:
+// quads of neurons per pair row.
+constexpr int ADJ_DENSE_Q = 4, ADJ_DENSE_TYPES = 4, ADJ_DENSE_THREADS = 384, ADJ_DENSE_NEURONS = 64;
+cudaError_t adj_dense_launch(const NetView &v, const AdjDenseView &av, int Q, int threads, int smem, long long step0,
+                             int nsteps, int n_types, float *grad_np, cudaStream_t stream);
+// Sum of the per-neuron parameter gradients into the neuron-type table.
+cudaError_t adj_reduce(const NetView &v, const double *gp_neuron, int n_types, float *grad_np, cudaStream_t stream);
+
 }  // namespace psst

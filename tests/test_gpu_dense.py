@@ -102,3 +102,36 @@ def test_dense_rows_agree_with_work_items(method):
                             ng.neuron_table(ng.HH), ng.synapse_table(ng.ACH))
     with psst.Network(dup) as net:
         assert net.info()["item_chunks"] > 0
+
+
+# sizes at the edges of the sweep's tiles: 32 neurons, 4 and 16 pair slots
+ADJ_SIZES = {
+    "small": [(2, 0.9, 1), (5, 0.8, 3), (16, 0.5, 2), (31, 0.3, 3)],
+    "32": [(32, 0.4, 1), (33, 0.3, 2), (63, 0.2, 1), (64, 0.2, 2)],
+    "128": [(96, 0.1, 1), (97, 0.15, 1), (127, 0.1, 1), (128, 0.5, 1)],
+}
+
+
+@pytest.mark.parametrize("method", ["rk4", "euler", "heun3"])
+@pytest.mark.parametrize("sizes", list(ADJ_SIZES))
+def test_dense_adjoint_matches_oracle(sizes, method):
+    # one batch of networks of uneven sizes, segments of uneven length, frames
+    # that fall inside and at the ends of segments; per-coordinate bound of the
+    # adjoint tests (1e-3, floor 1e-2 of the largest)
+    import torch
+    from paper_1906_03958_gb300 import psst
+    from tests.helpers import grad_error
+    spec = ng.concat_specs([_network(n, 700 + k, p, t) for k, (n, p, t) in enumerate(ADJ_SIZES[sizes])])
+    N, nsteps, stride = spec.n_neurons, 90, 3
+    g = np.random.default_rng(3).standard_normal((nsteps // stride, N))
+    tab = ([1 / 3, 2 / 3], [0.25, 0.0, 0.75])
+    kw = dict(order=1) if method == "euler" else dict(tableau=tab) if method == "heun3" else {}
+    gy64, gw64, gp64 = oracle.adjoint(spec, oracle.rest_state(spec), nsteps, g, stride, ckpt=30, **kw)
+    kw = dict(method=psst.METHOD_EULER) if method == "euler" else dict(tableau=tab) if method == "heun3" else {}
+    with psst.Network(spec, rec_stride=stride, rec_capacity=nsteps // stride, **kw) as net:
+        for ck in (40, 90, 7):
+            gw, gp, gy = (x.cpu().numpy() for x in net.adjoint(nsteps, torch.from_numpy(g.astype(np.float32)).cuda(), ck))
+            net.status()
+            assert grad_error(gw, gw64) <= 1e-3
+            assert grad_error(gp, gp64) <= 1e-3
+            assert grad_error(gy.ravel(), gy64[:4 * N]) <= 1e-3
