@@ -370,7 +370,7 @@ int smem_caps(int dev, SmemCaps *c) {
         cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess)
         return fail(PSST_ERR_CUDA, "cannot query shared memory sizes of device %d", dev);
-    const int stat = psst::cta_static_smem() + 64;  // static table + small shared variables
+    const int stat = psst::cta_static_smem() + 32;  // static table + small shared variables
     c->max_dyn = optin - stat;
     c->per_sm = per_sm;
     c->per_cta = stat + reserved;

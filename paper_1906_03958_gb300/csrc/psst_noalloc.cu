@@ -241,7 +241,7 @@ extern "C" int psst_integrate_grid_noalloc(const psst_device_network *d, int64_t
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
         return err_msg(PSST_ERR_CUDA, "device attributes");
-    const int max_dyn = optin - psst::cta_static_smem() - 64;
+    const int max_dyn = optin - psst::cta_static_smem() - 32;
     const int G = (int)std::max(1LL, std::min<long long>(std::min(sms, kMaxGrid), (N + 7) / 8));
     cudaStream_t st = (cudaStream_t)stream;
 
