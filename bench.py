@@ -123,8 +123,10 @@ def measured_peaks():
 # Sources that decide each kernel's memory traffic: its own file, the
 # shared device headers and the host planner (launch shapes, layouts).
 KERNEL_SOURCES = {
+    "dense_kernel": ("psst_dense.cu", "psst_dense.cuh", "psst_syn.cuh"),
     "net_kernel": ("psst_cta.cu", "psst_syn.cuh"),
     "grid_kernel": ("psst_grid.cu", "psst_syn.cuh"),
+    "adj_dense_kernel": ("psst_adjdense.cu", "psst_dense.cuh", "psst_syn.cuh"),
     "adj_kernel": ("psst_adjoint.cu",),
     "indep_kernel": ("psst_indep.cu",),
 }
@@ -532,7 +534,7 @@ def main():
         pairs = start.n_neurons * start.syn_params.shape[0]
         aflop = (ADJ_FLOP_SYN_STEP * start.n_synapses + ADJ_FLOP_NEURON_STEP * start.n_neurons
                  + ADJ_FLOP_PAIR_STEP * pairs) * T
-        atraffic = traffic_for("adj_kernel", "differentiated", T)
+        atraffic = traffic_for("adj_dense_kernel", "differentiated", T)
         adjoint = {"workload": f"64 antennal-lobe parameter sets, dense 120x120 W + GABA_B, {T} steps, "
                                f"checkpoint every {args.ckpt_every} (recorded by the forward), segment recompute",
                    "forward_ms": fwd_ms, "adjoint_ms": adj_ms, "ratio": adj_ms / fwd_ms,
@@ -540,7 +542,7 @@ def main():
                                 "peak": fp32_peak_tflops(smax), "unit": "TFLOP/s",
                                 "frac": aflop / (adj_ms / 1e3) / 1e12 / fp32_peak_tflops(smax),
                                 "traffic": atraffic,
-                                "kernel": "adj_kernel (one launch: segment recompute and reverse sweep)",
+                                "kernel": "adj_dense_kernel (one launch: segment recompute and reverse sweep)",
                                 "flop_per_step": {"synapse": ADJ_FLOP_SYN_STEP, "neuron": ADJ_FLOP_NEURON_STEP,
                                                   "neuron_type_pair": ADJ_FLOP_PAIR_STEP}}}
 
@@ -556,8 +558,8 @@ def main():
     dur = t_local / args.steps
     roof = {"bound": "alu", "achieved": flops_call / dur / 1e12, "peak": peak_tflops, "unit": "TFLOP/s",
             "frac": flops_call / dur / 1e12 / peak_tflops,
-            "traffic": traffic_for("net_kernel", args.workload),
-            "kernel": f"net_kernel: the {info['n_launch_classes']} size-class launches of one integrate call",
+            "traffic": traffic_for("dense_kernel", args.workload),
+            "kernel": f"dense_kernel: the {info['n_launch_classes']} size-class launches of one integrate call",
             "gates": "per (presynaptic neuron, type) pair" if pair_gates else "per synapse",
             "peak_source": f"FP32 FMA pipes: {n_sms} SMs x {FP32_LANES_PER_SM} lanes x 2 x "
                            f"{smax:.0f} MHz (sm_max_mhz of MEASURED_PEAKS.json)"}

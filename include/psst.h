@@ -190,7 +190,9 @@ int psst_create_network(const psst_network_desc *d, const psst_allocator *a, pss
    (Knuth's TwoSum; the handle keeps the remainders between calls), so the
    FP32 trajectory tracks the exact RK4 map far more closely than plain
    FP32 accumulation.  Asynchronous on `stream`;
-   device-side failures (NONFINITE, TIMEOUT) are reported by psst_status.
+   device-side failures (NONFINITE, TIMEOUT) are reported by psst_status
+   (once a network holds a NaN or infinity, the values of its other neurons
+   are unspecified; other networks of the batch are not affected).
    With the environment variable PSST_SYNC set (to anything but "0") the
    call synchronises `stream` and returns what psst_status would.
    n_steps = 0 is a no-op.  Errors: INVALID_ARG (n_steps < 0), CUDA. */

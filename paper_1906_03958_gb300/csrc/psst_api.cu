@@ -732,7 +732,7 @@ int setup_grid(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
         if (e == cudaSuccess) e = h->alloc(&g.flag, (size_t)parts * psst::GRID_FLAG_STRIDE);
         if (e == cudaSuccess && g.tix) {
             g.gts = g.used + parts;
-            e = h->alloc(&g.gt, (size_t)2 * g.gts);
+            e = h->alloc(&g.gt, (size_t)3 * g.gts);
         }
         g.row_split = rs;
         g.items = itd;

@@ -21,11 +21,16 @@
 // and no fence or flag sits between writer and reader: each CTA copies the
 // whole table into shared memory as the words arrive and gathers its
 // synapses' gates from there, instead of gathering an 8-byte map per
-// synapse from L2.  Each CTA also writes one tagged heartbeat word per
-// stage, after its own copy of the previous table, so that a CTA which has
-// seen every word of a phase knows that every CTA is done reading the
-// buffer it is about to overwrite (double buffering, as for the maps).
-// Both buffers are zeroed before each launch (phases start at 1).  Results
+// synapse from L2.  A pair's gate at stage s + 1 needs its neuron's potential
+// at stage s only, so it is published at the start of stage s and travels
+// while that stage's table copy, sums and potentials run (published at the
+// stage's end, every stage waited for the slowest CTA's words: 10,000 neurons
+// 20.1 -> 15.6 us per step, 3,764 12.4 -> 10.1, 1,800 9.7 -> 9.1).
+// Each CTA also writes one tagged heartbeat word per stage, after its own copy
+// of the stage's table.  Three tables, by phase modulo 3: the words of phase
+// q + 1 overwrite those of phase q - 2 by a CTA that has gathered phase q - 1,
+// whose heartbeats say that every CTA has copied phase q - 2.
+// The tables are zeroed before each launch (phases start at 1).  Results
 // are bitwise equal to the per-synapse variant.
 //
 // The per-synapse variant reads its maps straight from L2 during the
@@ -126,7 +131,7 @@ __device__ bool grid_gather(const GridView &g, unsigned long long phase, int *er
 
 // A gate-table word: phase tag (high half), value (low half).  Tags are
 // the phase modulo 2^32; a word read for phase q was last written for
-// phase q - 2 (or zeroed), so the wrap never makes a stale word match.
+// phase q - 3 (or zeroed), so the wrap never makes a stale word match.
 __device__ __forceinline__ unsigned long long gate_word(unsigned long long phase, float G) {
     return ((unsigned long long)(unsigned)phase << 32) | __float_as_uint(G);
 }
@@ -187,47 +192,78 @@ struct GlobalCoef {
 
 // One stage sg of the handle's method (a compile-time StageCT for the
 // classic RK4 stages, else a run-time StageRT: one copy of this code serves
-// every stage of Euler and a tableau); sx is the stage after it;
-// par selects the double-buffered potentials, gates and global tables this
-// stage reads (the parity of the stage's index counted over the launch).  On
-// entry the owned neurons' gates m, h, n of this stage are done and `phase`
-// is the phase every CTA must have published; on return the CTA has
-// published the next phase (phase updated) and, when `more`, computed the
-// next stage's (sx's) gates.
-template <bool HAS2, bool PAIR, class SG, class SX>
-__device__ __forceinline__ bool grid_stage(const NetView &v, const GridView &g, const SG &sg, const SX &sx,
-                                           const Items &it, int lo, int N, int nt, int M,
-                                           long long rec_slot, float *vst, float *y0, float *ylo, float *acc,
-                                           float *ys,
-                                           const float *prm, const float *iext, float2 *cur1, float2 *acc1,
-                                           float4 *cur2, float4 *acc2, float *pst, float *gtab, const float *stab,
-                                           int par, unsigned long long &phase, bool more, int *s_fail) {
+// every stage of Euler and a tableau); par selects the double-buffered
+// potentials, gates and per-synapse map tables this stage reads (the parity of
+// the stage's index counted over the launch), tab the gate table (phase mod
+// 3).  On entry `phase` is the phase every CTA must have published; on return
+// (phase updated) the CTA has published the next one.
+template <bool HAS2, bool PAIR, class SG>
+__device__ __forceinline__ bool grid_stage(const NetView &v, const GridView &g, const SG &sg, const Items &it, int lo,
+                                           int N, int nt, int M, long long rec_slot, float *vst, float *y0, float *ylo,
+                                           float *acc, float *ys, const float *prm, const float *iext, float2 *cur1,
+                                           float2 *acc1, float4 *cur2, float4 *acc2, float *pst, float *gtab,
+                                           const float *stab, int par, int &tab, unsigned long long &phase, int *s_fail) {
     const bool LAST = sg.last;
     const int tid = threadIdx.x, nthr = blockDim.x, Mloc = N * nt;
     const float *vcur = vst + par * N;
     float *vnxt = vst + (par ^ 1) * N;
     const float *ysc = ys + par * 3 * N;
     float *ysn = ys + (par ^ 1) * 3 * N;
+    const int tab_next = tab == 2 ? 0 : tab + 1;
+    unsigned long long *gout = PAIR ? g.gt + (size_t)tab_next * g.gts : nullptr;
+    if (PAIR) {
+        // gates of the own used pairs for the next stage (same operations as
+        // the per-synapse path): they need this stage's potentials only, so
+        // they are published before this stage's own wait and sums, and reach
+        // the other CTAs while these run
+        float *r0p = pst, *s0p = pst + Mloc, *r0lo = pst + 2 * Mloc, *s0lo = pst + 3 * Mloc;
+        for (int p = tid; p < Mloc; p += nthr) {
+            const int t = __ldg(g.tix + (size_t)lo * nt + p);
+            if (t < 0) continue;
+            float2 f1;
+            float4 f2 = make_float4(0.f, 0.f, 0.f, 0.f), d4 = f2;
+            float4 &c2 = HAS2 ? cur2[p] : d4;
+            float4 &a2 = HAS2 ? acc2[p] : d4;
+            const float *sp = stab + (p % nt) * ST_COLS;
+            coef_update<HAS2>(sp, vcur[p / nt], sg, cur1[p], acc1[p], f1, c2, a2, f2);
+            const bool sec = HAS2 && sp[SP_KIND] != 0.0f;
+            float G;
+            if (!LAST) {
+                G = pair_gate(sec, cur1[p], c2, r0p[p], s0p[p], r0lo[p], s0lo[p]);
+            } else {
+                // the step's end gates: the next step's first-stage gates and step-start state
+                float r0 = r0p[p], s0 = s0p[p], rl = r0lo[p], sl = s0lo[p];
+                pair_step(sec, f1, f2, r0, s0, rl, sl);
+                G = pair_gate(sec, make_float2(0.0f, 0.0f), make_float4(0.0f, 0.0f, 0.0f, f2.w), r0, s0, rl, sl);
+                r0p[p] = r0;
+                s0p[p] = s0;
+                r0lo[p] = rl;
+                s0lo[p] = sl;
+            }
+            st_relaxed64(gout + t, gate_word(phase + 1, G));
+        }
+    }
+    // the owned neurons' gates of this stage (own data) while the other CTAs finish
+    for (int i = nthr - 1 - tid; i < N; i += nthr) neuron_gates(sg, i, N, vcur[i], ysc, ysn, y0, ylo, acc);
     // the other CTAs' gates and maps of this stage are published (per pair:
     // this stage's gate of every used pair, copied as each owner's flag shows it)
     if (PAIR) {
-        if (!grid_gather_table(g, phase, g.gt + (size_t)par * g.gts, gtab, v.err, s_fail)) return false;
+        if (!grid_gather_table(g, phase, g.gt + (size_t)tab * g.gts, gtab, v.err, s_fail)) return false;
+        // this CTA is done reading that table: its heartbeat for the next phase
+        if (tid == 0) st_relaxed64(gout + g.used + blockIdx.x, gate_word(phase + 1, 0.0f));
         sphase_pair(it, gtab, 0);
     } else {
         if (!grid_gather(g, phase, v.err, s_fail)) return false;
         sphase<HAS2>(sg.first, it, GlobalCoef{g.c1 + (size_t)par * M, HAS2 ? g.c2 + (size_t)par * M : nullptr});
     }
     __syncthreads();
-    // independent work units: potential of each owned neuron and the gate map
-    // of each own (neuron, type) pair; the potentials take whole warps
-    float *r0p = pst, *s0p = pst + Mloc, *r0lo = pst + 2 * Mloc, *s0lo = pst + 3 * Mloc;
-    unsigned long long *gout = PAIR ? g.gt + (size_t)(par ^ 1) * g.gts : nullptr;
-    // this CTA is done reading the other table: its heartbeat for the next phase
-    if (PAIR && tid == 0) st_relaxed64(gout + g.used + blockIdx.x, gate_word(phase + 1, 0.0f));
+    // independent work units: potential of each owned neuron and (per-synapse
+    // layout) the gate map of each own (neuron, type) pair; the potentials
+    // take whole warps
     float2 *o1 = g.c1 + (size_t)(par ^ 1) * M + (size_t)lo * nt;
     float4 *o2 = HAS2 ? g.c2 + (size_t)(par ^ 1) * M + (size_t)lo * nt : nullptr;
     const int nw = (N + 31) & ~31;
-    const int U = nw + Mloc;
+    const int U = PAIR ? nw : nw + Mloc;
     for (int u = tid; u < U; u += nthr) {
         if (u < nw) {
             // the whole warp takes this branch (nw and nthr are multiples of 32)
@@ -242,45 +278,17 @@ __device__ __forceinline__ bool grid_stage(const NetView &v, const GridView &g, 
             const float vn = neuron_v_post(sg, i, pre, isyn, y0, ylo, acc);
             vnxt[i] = vn;
             if (LAST && rec_slot >= 0) v.rec[rec_slot * v.N + lo + i] = vn;
-        } else {
+        } else if (!PAIR) {
+            // gate map of an own pair: local copy for the next stage, and the
+            // table every CTA reads at the next stage
             const int p = u - nw;
-            if (PAIR) {
-                // gate of an own used pair for the next stage (same operations as
-                // the per-synapse path), published in the other table
-                const int t = __ldg(g.tix + (size_t)lo * nt + p);
-                if (t < 0) continue;
-                float2 f1;
-                float4 f2 = make_float4(0.f, 0.f, 0.f, 0.f), d4 = f2;
-                float4 &c2 = HAS2 ? cur2[p] : d4;
-                float4 &a2 = HAS2 ? acc2[p] : d4;
-                const float *sp = stab + (p % nt) * ST_COLS;
-                coef_update<HAS2>(sp, vcur[p / nt], sg, cur1[p], acc1[p], f1, c2, a2, f2);
-                const bool sec = HAS2 && sp[SP_KIND] != 0.0f;
-                float G;
-                if (!LAST) {
-                    G = pair_gate(sec, cur1[p], c2, r0p[p], s0p[p], r0lo[p], s0lo[p]);
-                } else {
-                    // the step's end gates: the next step's first-stage gates and step-start state
-                    float r0 = r0p[p], s0 = s0p[p], rl = r0lo[p], sl = s0lo[p];
-                    pair_step(sec, f1, f2, r0, s0, rl, sl);
-                    G = pair_gate(sec, make_float2(0.0f, 0.0f), make_float4(0.0f, 0.0f, 0.0f, f2.w), r0, s0, rl, sl);
-                    r0p[p] = r0;
-                    s0p[p] = s0;
-                    r0lo[p] = rl;
-                    s0lo[p] = sl;
-                }
-                st_relaxed64(gout + t, gate_word(phase + 1, G));
-            } else {
-                // gate map of an own pair: local copy for the next stage, and the
-                // table every CTA reads at the next stage
-                float2 f1;
-                float4 f2 = make_float4(0.f, 0.f, 0.f, 0.f), d4 = f2;
-                float4 &c2 = HAS2 ? cur2[p] : d4;
-                float4 &a2 = HAS2 ? acc2[p] : d4;
-                coef_update<HAS2>(stab + (p % nt) * ST_COLS, vcur[p / nt], sg, cur1[p], acc1[p], f1, c2, a2, f2);
-                o1[p] = LAST ? f1 : cur1[p];
-                if (HAS2) o2[p] = LAST ? f2 : cur2[p];
-            }
+            float2 f1;
+            float4 f2 = make_float4(0.f, 0.f, 0.f, 0.f), d4 = f2;
+            float4 &c2 = HAS2 ? cur2[p] : d4;
+            float4 &a2 = HAS2 ? acc2[p] : d4;
+            coef_update<HAS2>(stab + (p % nt) * ST_COLS, vcur[p / nt], sg, cur1[p], acc1[p], f1, c2, a2, f2);
+            o1[p] = LAST ? f1 : cur1[p];
+            if (HAS2) o2[p] = LAST ? f2 : cur2[p];
         }
     }
     if (PAIR) {
@@ -289,13 +297,7 @@ __device__ __forceinline__ bool grid_stage(const NetView &v, const GridView &g, 
     } else {
         grid_publish(g, ++phase);
     }
-    if (more) {
-        // the next stage's gates of the owned neurons (own data only) while
-        // the other CTAs finish; that stage reads this one's ysn and vnxt
-        // (after a step's last stage comes the first stage of the next step)
-        float *ysx = ys + par * 3 * N;
-        for (int i = nthr - 1 - tid; i < N; i += nthr) neuron_gates(sx, i, N, vnxt[i], ysn, ysx, y0, ylo, acc);
-    }
+    tab = tab_next;
     return true;
 }
 
@@ -350,7 +352,7 @@ __device__ void grid_run(const NetView &v, const GridView &g, long long step0, i
     const long long pon = v.pulse_on[0], poff = v.pulse_off[0];
     if (PAIR) {
         // own pairs' step-start gates from one synapse of each, and their
-        // stage-0 gates (identity step-end map) in table 0
+        // stage-0 gates (identity step-end map) in table 1
         float *r0p = pst, *s0p = pst + Mloc, *r0lo = pst + 2 * Mloc, *s0lo = pst + 3 * Mloc;
         for (int p = tid; p < Mloc; p += nthr) {
             const int t = g.tix[(size_t)lo * nt + p];
@@ -367,7 +369,7 @@ __device__ void grid_run(const NetView &v, const GridView &g, long long step0, i
                 }
                 const float G0 = pair_gate(sec, make_float2(0.0f, 0.0f),
                                            make_float4(0.0f, 0.0f, 0.0f, sec ? sp[SP_KD] : 1.0f), r0, s0, rl, sl);
-                st_relaxed64(g.gt + t, gate_word(1, G0));
+                st_relaxed64(g.gt + g.gts + t, gate_word(1, G0));  // table 1 (phase 1)
             }
             r0p[p] = r0;
             s0p[p] = s0;
@@ -393,21 +395,13 @@ __device__ void grid_run(const NetView &v, const GridView &g, long long step0, i
     // identity maps behind a flag)
     unsigned long long phase = 1;
     if (PAIR) {
-        if (tid == 0) st_relaxed64(g.gt + g.used + blockIdx.x, gate_word(1, 0.0f));
+        if (tid == 0) st_relaxed64(g.gt + g.gts + g.used + blockIdx.x, gate_word(1, 0.0f));
         __syncthreads();
     } else {
         grid_publish(g, phase);
     }
-    // the first stage's gates (own data) while the other CTAs finish setting up
-    {
-        const float *ysc = ys, *vcur = vst;
-        float *ysn = ys + 3 * N;
-        if (nsteps > 0) {
-            const StageRT s0 = stage_rt(v, 0, dt);
-            for (int i = nthr - 1 - tid; i < N; i += nthr) neuron_gates(s0, i, N, vcur[i], ysc, ysn, y0, ylo, acc);
-        }
-    }
     bool ok = true;
+    int tab = 1;  // gate table of the phase: phase mod 3
     // record: phase of (step + 1) modulo the stride, advanced once per step
     int rec_phase = v.rec_stride > 0 ? (int)((step0 + 1) % v.rec_stride) : -1;
     for (int itn = 0; ok && itn < nsteps; ++itn) {
@@ -420,26 +414,18 @@ __device__ void grid_run(const NetView &v, const GridView &g, long long step0, i
         }
         for (int i = tid; i < N; i += nthr)
             iext[i] = input_current(v, inp[i], inp[N + i], in_pulse, (long long)lo + i, step);
-        const bool more = itn + 1 < nsteps;
         // stage s of step itn reads parity (itn * ns + s) & 1
-#define PSST_GSTAGE(SG, SX, par, mo)                                                                            \
-    grid_stage<HAS2, PAIR>(v, g, SG, SX, it, lo, N, nt, M, rec_slot, vst, y0, ylo, acc, ys, prm, iext, cur1, acc1, \
-                           cur2, acc2, pst, gtab, stab, par, phase, mo, s_fail)
+#define PSST_GSTAGE(SG, par)                                                                                        \
+    grid_stage<HAS2, PAIR>(v, g, SG, it, lo, N, nt, M, rec_slot, vst, y0, ylo, acc, ys, prm, iext, cur1, acc1, cur2, \
+                           acc2, pst, gtab, stab, par, tab, phase, s_fail)
         if (v.method == PSST_METHOD_RK4) {
-            const StageCT<0> k0{stage_coef<0>(v, dt)};
-            const StageCT<1> k1{stage_coef<1>(v, dt)};
-            const StageCT<2> k2{stage_coef<2>(v, dt)};
-            const StageCT<3> k3{stage_coef<3>(v, dt)};
-            ok = PSST_GSTAGE(k0, k1, 0, true);
-            if (ok) ok = PSST_GSTAGE(k1, k2, 1, true);
-            if (ok) ok = PSST_GSTAGE(k2, k3, 0, true);
-            if (ok) ok = PSST_GSTAGE(k3, k0, 1, more);
+            ok = PSST_GSTAGE(StageCT<0>{stage_coef<0>(v, dt)}, 0);
+            if (ok) ok = PSST_GSTAGE(StageCT<1>{stage_coef<1>(v, dt)}, 1);
+            if (ok) ok = PSST_GSTAGE(StageCT<2>{stage_coef<2>(v, dt)}, 0);
+            if (ok) ok = PSST_GSTAGE(StageCT<3>{stage_coef<3>(v, dt)}, 1);
         } else {
 #pragma unroll 1
-            for (int s = 0; ok && s < ns; ++s) {
-                const StageRT sg = stage_rt(v, s, dt), sx = stage_rt(v, s + 1 < ns ? s + 1 : 0, dt);
-                ok = PSST_GSTAGE(sg, sx, (itn * ns + s) & 1, s + 1 < ns || more);
-            }
+            for (int s = 0; ok && s < ns; ++s) ok = PSST_GSTAGE(stage_rt(v, s, dt), (itn * ns + s) & 1);
         }
 #undef PSST_GSTAGE
         // the next step's input currents (own data) run before stage 0's wait
@@ -524,7 +510,7 @@ cudaError_t grid_occupancy(int block, int smem, int *blocks_per_sm) {
 cudaError_t grid_launch(const NetView &v, const GridView &g, long long step0, int nsteps, int grid, int block,
                         int smem, cudaStream_t stream) {
     cudaError_t e = cudaMemsetAsync(g.flag, 0, (size_t)grid * GRID_FLAG_STRIDE * sizeof(unsigned long long), stream);
-    if (e == cudaSuccess && g.pair) e = cudaMemsetAsync(g.gt, 0, 2 * (size_t)g.gts * sizeof(unsigned long long), stream);
+    if (e == cudaSuccess && g.pair) e = cudaMemsetAsync(g.gt, 0, 3 * (size_t)g.gts * sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return e;
     void *args[] = {(void *)&v, (void *)&g, (void *)&step0, (void *)&nsteps};
     return cudaLaunchCooperativeKernel((const void *)grid_kernel, dim3(grid), dim3(block), args, (size_t)smem,
