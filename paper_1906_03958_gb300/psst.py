@@ -129,10 +129,27 @@ def _check(rc: int):
         raise PsstError(rc, load().psst_last_error().decode())
 
 
+_current_stream = None
+
+
+def _stream_getter():
+    """A function returning the raw handle of the current torch stream:
+    torch's own raw query where it has one (0.3 us a call instead of 2.5 for
+    building a Stream object, in calls that launch one short kernel)."""
+    import torch
+    torch.cuda.current_stream()  # initialises CUDA
+    raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or dev is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(dev())
+
+
 def _stream_handle(stream):
+    global _current_stream
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        if _current_stream is None:
+            _current_stream = _stream_getter()
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -236,6 +253,7 @@ class Network:
         _check(lib.psst_create_network(C.byref(d), C.byref(self._allocator.struct) if self._allocator else None,
                                        C.byref(h)))
         self._h = h
+        self._lib = lib
         self.device = device
         self.N = spec.n_neurons
         self.S = spec.n_synapses
@@ -267,7 +285,7 @@ class Network:
 
     # -- stepping
     def integrate(self, n_steps: int, stream=None):
-        _check(load().psst_integrate(self._h, int(n_steps), _stream_handle(stream)))
+        _check(self._lib.psst_integrate(self._h, int(n_steps), _stream_handle(stream)))
 
     def status(self, stream=None):
         _check(load().psst_status(self._h, _stream_handle(stream)))
@@ -290,13 +308,14 @@ class Network:
     def get_state(self, out=None, stream=None):
         """State [V, m, h, n, r, s] into ``out`` (CUDA tensor or numpy array);
         default: a new float32 CUDA tensor."""
-        import torch
         if out is None:
+            import torch
             out = torch.empty(self.dim, dtype=torch.float32, device=f"cuda:{self.device}")
-        on_dev = isinstance(out, torch.Tensor) and out.is_cuda
-        ptr = out.data_ptr() if isinstance(out, torch.Tensor) else out.ctypes.data
-        n = out.numel() if isinstance(out, torch.Tensor) else out.size
-        _check(load().psst_get_state(self._h, ptr, n, int(on_dev), _stream_handle(stream)))
+        if isinstance(out, np.ndarray):
+            on_dev, ptr, n = 0, out.ctypes.data, out.size
+        else:
+            on_dev, ptr, n = int(out.is_cuda), out.data_ptr(), out.numel()
+        _check(self._lib.psst_get_state(self._h, ptr, n, on_dev, _stream_handle(stream)))
         return out
 
     def get_state_numpy(self) -> np.ndarray:
