@@ -444,10 +444,12 @@ __device__ void sweep_run(const NetView &v, const AdjDenseView &av, const AdjDen
                         yp = ys = make_float2(0.0f, 0.0f);
                         copy_wait();
                     }
-                    bar_all();
+                    // (read before the barrier: the next step's copy into this
+                    // buffer may start as soon as one warp has passed it)
                     float G[4];
 #pragma unroll
                     for (int r = 0; r < 4; ++r) G[r] = F1(pb + 16 * (s0 + r) + 12);
+                    bar_all();
 #pragma unroll
                     for (int q = 0; q < Q; ++q) {
                         const float4 z = F4(z1 + 128 * q);
