@@ -56,9 +56,10 @@ __device__ __forceinline__ unsigned cluster_rank() {
     return r;
 }
 
+// (Without .aligned, for the same reason as bar_all below.)
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 __device__ __forceinline__ void copy16(int o, const float4 *src) {
@@ -69,8 +70,10 @@ __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_gr
 __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // The CTA's barrier, met by the sweep's pair warps and neuron warps at
-// different places of their code.
-__device__ __forceinline__ void bar_all() { asm volatile("bar.sync 0;" ::: "memory"); }
+// different places of their code.  (barrier.sync, not bar.sync, which is the
+// aligned form: lanes without a neuron or past a copy's end need not have
+// reconverged with the others of their warp.)
+__device__ __forceinline__ void bar_all() { asm volatile("barrier.sync 0;" ::: "memory"); }
 
 // ---------------------------------------------------------------- recompute
 

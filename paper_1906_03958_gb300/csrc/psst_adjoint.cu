@@ -74,10 +74,11 @@ __device__ __forceinline__ unsigned cluster_rank() {
 }
 
 // Barrier of the cluster's CTAs; release/acquire orders their global memory
-// accesses across it.
+// accesses across it.  (Without .aligned: defined for lanes of a warp that
+// have not reconverged.)
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 struct AdjSmem {

@@ -54,9 +54,11 @@ __device__ __forceinline__ unsigned cluster_rank() {
     return r;
 }
 
+// (Without .aligned: warps arrive from loops whose lanes leave at different
+// times, and only this form is defined for lanes that have not reconverged.)
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 __device__ __forceinline__ void st_peer(float *local, unsigned rank, float x) {

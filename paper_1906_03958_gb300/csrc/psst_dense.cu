@@ -56,8 +56,10 @@ __device__ __forceinline__ unsigned cluster_rank() {
     return r;
 }
 
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// (Without .aligned: warps arrive from loops whose lanes leave at different
+// times, and only this form is defined for lanes that have not reconverged.)
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
 // x into the float at offset o of every CTA of the cluster.
 __device__ __forceinline__ void put(int o, int cl, float x) {
