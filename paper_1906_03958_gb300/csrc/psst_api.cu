@@ -96,7 +96,7 @@ struct psst_net {
     int max_dyn = 0;
     SmemCaps caps{};
     // adjoint plan and scratch (allocated on the first psst_adjoint)
-    std::vector<int> adj_K, adj_items;
+    std::vector<int> adj_K;  // empty: not planned
     int adj_smem = 0;
     int *d_adjK = nullptr, *d_adjI = nullptr, *d_adjKC = nullptr, *d_adjCI = nullptr;
     int *d_cib = nullptr, *d_ck = nullptr;  // column plan: items of each pair, synapse of each slot
@@ -165,8 +165,18 @@ struct psst_net {
             e = cudaMalloc(&q, bytes);
         }
         if (e == cudaSuccess) allocs.push_back(q);
+        else cudaGetLastError();  // reported here, not by a later launch's check
         *p = (T *)q;
         return e;
+    }
+    // Give one block back.  No work that uses it may be in flight.
+    template <class T>
+    void drop(T *&p) {
+        if (!p) return;
+        allocs.erase(std::find(allocs.begin(), allocs.end(), (void *)p));
+        if (user_alloc.free) user_alloc.free((void *)p, user_alloc.ctx);
+        else cudaFree((void *)p);
+        p = nullptr;
     }
     // CTA mode: one stream per size class; an integrate call forks them off
     // the caller's stream and joins them back, so the classes' launches run
@@ -1696,6 +1706,15 @@ int psst_set_neuron_params(psst_net *h, const float *p, size_t n, int on_device,
     return e == cudaSuccess ? PSST_OK : cuda_fail(e, "psst_set_neuron_params");
 }
 
+// Give back what the adjoint over dense rows alone uses.
+static void drop_adj_dense(psst_net *h) {
+    h->drop(h->d_adjd_plans);
+    h->drop(h->d_adjd_pair);
+    h->drop(h->d_adjd_slot);
+    h->drop(h->d_adjd_col);
+    h->drop(h->adjd_gtot);
+}
+
 // Plan of the adjoint over dense rows (psst_adjdense.cu): for handles whose
 // networks all have at most 128 neurons, 4 synapse types, 160 slots of used
 // pairs and no two synapses of one pair in a row.
@@ -1758,6 +1777,7 @@ static int plan_adj_dense(psst_net *h) {
     if (e == cudaSuccess && !h->adj_gpn) e = h->alloc(&h->adj_gpn, (size_t)h->v.N * 9);
     if (e == cudaSuccess && !h->adj_gy0) e = h->alloc(&h->adj_gy0, (size_t)h->v.N * 4);
     if (e != cudaSuccess) {
+        drop_adj_dense(h);
         h->adjd_state = 0;
         return cuda_fail(e, "psst_adjoint buffers");
     }
@@ -1768,6 +1788,19 @@ static int plan_adj_dense(psst_net *h) {
     h->adjd_span = -1;
     h->adjd_state = 1;
     return PSST_OK;
+}
+
+// Segment buffers of at least `floats` floats.  On failure the present ones
+// stay, with the plans laid out for them; on success they stay allocated too
+// (an earlier call's kernel may still use them).
+static cudaError_t grow_segments(psst_net *h, long long floats) {
+    if (floats <= h->adj_seg_cap) return cudaSuccess;
+    float *seg = nullptr;
+    const cudaError_t e = h->alloc(&seg, (size_t)floats);
+    if (e != cudaSuccess) return e;
+    h->adj_seg = seg;
+    h->adj_seg_cap = floats;
+    return cudaSuccess;
 }
 
 // The adjoint over dense rows of the recorded span.
@@ -1782,13 +1815,10 @@ static int adjoint_dense(psst_net *h, long long s0, int n_steps, int ckpt_every,
             p.seg_off = total;
             total += 2 * span * ns * psst::adj_stage_floats(h->pin.net_off[b + 1] - h->pin.net_off[b], p.Mp);
         }
-        cudaError_t e = cudaSuccess;
-        if (total > h->adj_seg_cap) {
-            e = h->alloc(&h->adj_seg, (size_t)total);
-            h->adj_seg_cap = e == cudaSuccess ? total : 0;
-        }
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(h->d_adjd_plans, h->adjd_plans.data(), h->adjd_plans.size() * sizeof(psst::AdjDensePlan),
+        cudaError_t e = grow_segments(h, total);
+        if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint storage");
+        h->adjd_span = -1;  // until the plans for it are there
+        e = cudaMemcpyAsync(h->d_adjd_plans, h->adjd_plans.data(), h->adjd_plans.size() * sizeof(psst::AdjDensePlan),
                                 cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint storage");
         h->adjd_span = span;
@@ -1885,8 +1915,7 @@ int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_fra
         std::vector<uint32_t> code((size_t)h->v.S);
         e = cudaMemcpy(code.data(), h->v.syn_code, code.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint plan");
-        h->adj_K.resize(n_nets);
-        h->adj_items.resize(n_nets);
+        std::vector<int> adj_K((size_t)n_nets), adj_items((size_t)n_nets);
         std::vector<int> KC((size_t)n_nets), citems((size_t)n_nets), cib, ck;
         std::vector<unsigned short> crow;
         std::vector<long long> cslot_off((size_t)n_nets), cib_off((size_t)n_nets);
@@ -1945,15 +1974,15 @@ int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_fra
                     ck[(size_t)slot] = (int)(k - sb);
                     crow[(size_t)slot] = (unsigned short)(i - n0);
                 }
-            h->adj_K[b] = K;
-            h->adj_items[b] = items;
+            adj_K[b] = K;
+            adj_items[b] = items;
             KC[b] = kc;
             citems[b] = nci;
             slots += cslots;
         }
         h->adj_smem = need;
-        e = upload(h, &h->d_adjK, h->adj_K.data(), h->adj_K.size());
-        if (e == cudaSuccess) e = upload(h, &h->d_adjI, h->adj_items.data(), h->adj_items.size());
+        e = upload(h, &h->d_adjK, adj_K.data(), adj_K.size());
+        if (e == cudaSuccess) e = upload(h, &h->d_adjI, adj_items.data(), adj_items.size());
         if (e == cudaSuccess) e = upload(h, &h->d_adjKC, KC.data(), KC.size());
         if (e == cudaSuccess) e = upload(h, &h->d_adjCI, citems.data(), citems.size());
         if (e == cudaSuccess) e = upload(h, &h->d_cib, cib.data(), cib.size());
@@ -1966,7 +1995,22 @@ int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_fra
         if (e == cudaSuccess && !h->adj_gpn) e = h->alloc(&h->adj_gpn, (size_t)h->v.N * 9);
         if (e == cudaSuccess && !h->adj_gy0) e = h->alloc(&h->adj_gy0, (size_t)h->v.N * 4);
         if (e == cudaSuccess) e = h->alloc(&h->d_segoff, (size_t)n_nets);
-        if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint buffers");
+        if (e != cudaSuccess) {
+            h->drop(h->d_adjK);
+            h->drop(h->d_adjI);
+            h->drop(h->d_adjKC);
+            h->drop(h->d_adjCI);
+            h->drop(h->d_cib);
+            h->drop(h->d_ciboff);
+            h->drop(h->d_ck);
+            h->drop(h->d_crow);
+            h->drop(h->d_cslotoff);
+            h->drop(h->adj_gpart);
+            h->drop(h->adj_gtot);
+            h->drop(h->d_segoff);
+            return cuda_fail(e, "psst_adjoint buffers");
+        }
+        h->adj_K = adj_K;  // planned: only now that every buffer is there
     }
     // checkpoint and segment storage for this span (grown on demand)
     {
@@ -1982,10 +2026,7 @@ int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_fra
             seg_total += 2LL * std::min<long long>(ckpt_every, n_steps) * step_floats;  // two buffers
         }
         h->adjd_span = -1;  // the buffer's layout is this path's now
-        if (seg_total > h->adj_seg_cap) {
-            e = h->alloc(&h->adj_seg, (size_t)seg_total);
-            h->adj_seg_cap = seg_total;
-        }
+        e = grow_segments(h, seg_total);
         if (e == cudaSuccess) e = cudaMemcpy(h->d_segoff, sg.data(), sg.size() * sizeof(long long), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint storage");
     }
