@@ -108,7 +108,7 @@ struct Recompute {
         }
         if (tid < ns) {
             const StageRT s = stage_rt(v, tid, v.dt);
-            F4(lay.sc + 16 * tid) = make_float4(s.c.w, s.c.cn, s.c.fin, 0.0f);
+            F4(lay.sc + 16 * tid) = make_float4(s.c.w, s.c.cn, s.c.fin, s.c.finl);
         }
         const int SR = pl.rows;  // a multiple of 4
         for (int r0 = 0; r0 < N; r0 += SR) {
@@ -191,7 +191,7 @@ struct Recompute {
         const long long pon = v.pulse_on[b], poff = v.pulse_off[b];
         int vc = lay.vst, vn = lay.vst + 4 * Nw, yc = lay.ys, yn = lay.ys + 16 * Nw, gc = lay.g, gn = lay.g + 4 * C;
         const float4 c0 = F4(lay.sc);
-        StageCoef cf{c0.x, c0.y, c0.z};
+        StageCoef cf{c0.x, c0.y, c0.z, c0.w};
         float iext = 0.0f;
         auto stage = [&](auto last, int next) {
             constexpr bool LAST = decltype(last)::value;
@@ -239,19 +239,16 @@ struct Recompute {
                 const int o = lay.gst + 16 * i;
                 float4 m = F4(o), h = F4(o + 16 * Nw), n = F4(o + 32 * Nw);
                 const float am = alpha_m(Vi, e), bm = beta_m(Vi), ah = alpha_h(Vi), bh = beta_h(e), an = alpha_n(Vi, e),
-                            bn = beta_n(Vi), dn = den_n(e);
+                            bn = beta_n(Vi);
                 if (i < N) {
-                    const float dam = 0.1f * ratio_u_deriv(__fmul_rn(__fadd_rn(Vi, 40.0f), 0.1f), am, e, __fsub_rn(1.0f, e));
-                    const float dan = 0.01f * ratio_u_deriv(__fmul_rn(__fadd_rn(Vi, 55.0f), 0.1f), 10.0f * an,
-                                                            __fsub_rn(1.0f, dn), dn);
                     *(float4 *)(rec + 4 * i) = make_float4(Vi, m.w, h.w, n.w);
                     float *ls = rec + 4 * N + 4 * i, *gd = rec + 8 * N + 4 * i;
                     ls[0] = am + bm;
                     ls[1] = ah + bh;
                     ls[2] = an + bn;
-                    gd[0] = dam * (1.0f - m.w) + bm * (1.0f / 18.0f) * m.w;
-                    gd[1] = -ah * (1.0f / 20.0f) * (1.0f - h.w) - bh * (1.0f - bh) * 0.1f * h.w;
-                    gd[2] = dan * (1.0f - n.w) + bn * (1.0f / 80.0f) * n.w;
+                    gd[0] = slope_m(Vi, e, am, bm, m.w);
+                    gd[1] = slope_h(ah, bh, h.w);
+                    gd[2] = slope_n(Vi, e, an, bn, n.w);
                 }
                 gate_update<LAST>(cf, am, bm, m);
                 gate_update<LAST>(cf, ah, bh, h);
@@ -281,7 +278,7 @@ struct Recompute {
                     acc = ac;
                     V = ext_stage(y0, ylo, cf.cn, d);
                 } else {
-                    ext_step(y0, ylo, cf.fin, ac);
+                    ext_step(y0, ylo, cf.fin, cf.finl, ac);
                     acc = 0.0f;
                     V = y0;
                 }
@@ -292,7 +289,7 @@ struct Recompute {
                 }
             }
             const float4 c4 = F4(lay.sc + 16 * next);
-            cf = StageCoef{c4.x, c4.y, c4.z};
+            cf = StageCoef{c4.x, c4.y, c4.z, c4.w};
             __syncthreads();
             int t = vc;
             vc = vn;

@@ -203,8 +203,7 @@ __device__ void fwd_step(const NetView &v, const AdjNet &a, const AdjSmem &S, co
         __syncthreads();
         const float WGT = TAB ? v.rk_w[st] : (st == 0 || st == 3) ? 1.0f : 2.0f;
         const float cnext = TAB ? (st < 3 ? v.rk_c[st] * dt : 0.0f) : (st == 2) ? dt : 0.5f * dt;
-        const float dt6 = TAB ? v.rk_beta * dt : NST == 1 ? dt : dt * (1.0f / 6.0f);  // scale of the step's sum
-        const float W0 = TAB ? v.rk_w[0] : 1.0f;  // weight of the first stage's slope
+        const float dt6 = v.fin, dt6l = v.finl;  // scale of the step's sum
         // independent units, each on its own thread: the potential of each
         // neuron (row sums, ionic current), its gates m, h, n (rate
         // functions) and every gate pair (transmitter, r and s)
@@ -230,12 +229,12 @@ __device__ void fwd_step(const NetView &v, const AdjNet &a, const AdjSmem &S, co
                     S.sA[st * N + i] = A;
                     S.sfv[st * N + i] = fV;
                 }
-                const float ac = (st == 0) ? W0 * fV : fmaf(WGT, fV, S.acc[i]);
+                const float ac = (st == 0) ? WGT * fV : fmaf(WGT, fV, S.acc[i]);
                 if (st < NST - 1) {
                     S.acc[i] = ac;
                     S.sV[(st + 1) * N + i] = ext_stage(S.y[i], S.ylo[i], cnext, fV);
                 } else {
-                    ext_step(S.y[i], S.ylo[i], dt6, ac);
+                    ext_step(S.y[i], S.ylo[i], dt6, dt6l, ac);
                 }
             } else if (u < 2 * N) {
                 const int i = u - N;
@@ -247,12 +246,12 @@ __device__ void fwd_step(const NetView &v, const AdjNet &a, const AdjSmem &S, co
 #pragma unroll
                 for (int x = 1; x < 4; ++x) {
                     const int ix = x * N + i;
-                    const float ac = (st == 0) ? W0 * d[x - 1] : fmaf(WGT, d[x - 1], S.acc[ix]);
+                    const float ac = (st == 0) ? WGT * d[x - 1] : fmaf(WGT, d[x - 1], S.acc[ix]);
                     if (st < NST - 1) {
                         S.acc[ix] = ac;
                         stg[x][(st + 1) * N + i] = ext_stage(S.y[ix], S.ylo[ix], cnext, d[x - 1]);
                     } else {
-                        ext_step(S.y[ix], S.ylo[ix], dt6, ac);
+                        ext_step(S.y[ix], S.ylo[ix], dt6, dt6l, ac);
                     }
                 }
             } else {
@@ -265,8 +264,8 @@ __device__ void fwd_step(const NetView &v, const AdjNet &a, const AdjSmem &S, co
                 const float dr = sp[SP_A] * T * (1.0f - rs) - sp[SP_B] * rs;
                 const float ds = sp[SP_KIND] != 0.0f ? sp[SP_K3] * rs - sp[SP_K4] * ss : 0.0f;
                 const int ir = 4 * N + p, is = 4 * N + M + p;
-                const float ar = (st == 0) ? W0 * dr : fmaf(WGT, dr, S.acc[ir]);
-                const float as = (st == 0) ? W0 * ds : fmaf(WGT, ds, S.acc[is]);
+                const float ar = (st == 0) ? WGT * dr : fmaf(WGT, dr, S.acc[ir]);
+                const float as = (st == 0) ? WGT * ds : fmaf(WGT, ds, S.acc[is]);
                 if (st < NST - 1) {
                     S.acc[ir] = ar;
                     S.acc[is] = as;
@@ -277,8 +276,8 @@ __device__ void fwd_step(const NetView &v, const AdjNet &a, const AdjSmem &S, co
                     const float s2 = sn * sn, s4 = s2 * s2;
                     S.sG[(st + 1) * M + p] = sp[SP_KIND] != 0.0f ? __fdiv_rn(s4, s4 + sp[SP_KD]) : rn;
                 } else {
-                    ext_step(S.y[ir], S.ylo[ir], dt6, ar);
-                    ext_step(S.y[is], S.ylo[is], dt6, as);
+                    ext_step(S.y[ir], S.ylo[ir], dt6, dt6l, ar);
+                    ext_step(S.y[is], S.ylo[is], dt6, dt6l, as);
                 }
             }
         }
@@ -361,33 +360,25 @@ __device__ void rev_step(const AdjNet &a, const AdjSmem &S, const float *stab, c
                 // gate x: its rate functions (those of hh_rates) and their derivatives
                 const int ix = x * N + i;
                 const float kbx = cb[st] * S.lam[ix] + (st < NST - 1 ? ca[st] * S.yprev[ix] : 0.0f);
-                float al, be, dal, dbe, g, yp;
+                float al, be, dg, yp;
                 const float e = rate_e(Vs);
                 if (x == 1) {
-                    const float u = __fmul_rn(__fadd_rn(Vs, 40.0f), 0.1f);
                     al = alpha_m(Vs, e);
                     be = beta_m(Vs);
-                    dal = 0.1f * ratio_u_deriv(u, al, e, __fsub_rn(1.0f, e));
-                    dbe = -be * (1.0f / 18.0f);
-                    g = ms;
+                    dg = slope_m(Vs, e, al, be, ms);
                     yp = -q * gNa * 3.0f * ms * ms * hs * (Vs - ENa);
                 } else if (x == 2) {
                     al = alpha_h(Vs);
                     be = beta_h(e);
-                    dal = -al * (1.0f / 20.0f);
-                    dbe = be * (1.0f - be) * 0.1f;
-                    g = hs;
+                    dg = slope_h(al, be, hs);
                     yp = -q * gNa * ms * ms * ms * (Vs - ENa);
                 } else {
-                    const float u = __fmul_rn(__fadd_rn(Vs, 55.0f), 0.1f), den = den_n(e);
                     al = alpha_n(Vs, e);
                     be = beta_n(Vs);
-                    dal = 0.01f * ratio_u_deriv(u, 10.0f * al, __fsub_rn(1.0f, den), den);
-                    dbe = -be * (1.0f / 80.0f);
-                    g = ns;
+                    dg = slope_n(Vs, e, al, be, ns);
                     yp = -q * gK * 4.0f * ns * ns * ns * (Vs - EK);
                 }
-                S.uvg[(x - 1) * N + i] = make_float2(kbx, dal * (1.0f - g) - dbe * g);
+                S.uvg[(x - 1) * N + i] = make_float2(kbx, dg);
                 S.yprev[ix] = yp - kbx * (al + be);
             }
         }

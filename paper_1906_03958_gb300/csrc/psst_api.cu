@@ -1104,6 +1104,7 @@ int psst_create_network(const psst_network_desc *d, const psst_allocator *a, pss
         for (int q = 0; q < 4; ++q) v.rk_w[q] = q < d->rk_stages ? d->rk_b[q] / v.rk_beta : 0.0f;
         for (int q = 0; q < 3; ++q) v.rk_c[q] = q + 1 < d->rk_stages ? d->rk_a[q] : 0.0f;
     }
+    psst::step_scale(v);
     v.rec_stride = d->rec_stride;
     v.rec_cap = d->rec_stride > 0 ? d->rec_capacity : 0;
 

@@ -115,7 +115,7 @@ __device__ __forceinline__ void dense_run(const NetView &v, const int b, const D
     const int ns = method_stages(v);
     if (tid < ns) {
         const StageRT s = stage_rt(v, tid, v.dt);
-        F4(lay.sc + 16 * tid) = make_float4(s.c.w, s.c.cn, s.c.fin, 0.0f);
+        F4(lay.sc + 16 * tid) = make_float4(s.c.w, s.c.cn, s.c.fin, s.c.finl);
     }
     const int SR = pl.stage_rows;  // a multiple of 4
     for (int r0 = 0; r0 < nown; r0 += SR) {
@@ -202,7 +202,7 @@ __device__ __forceinline__ void dense_run(const NetView &v, const int b, const D
     int gc = lay.g, gn = lay.g + 4 * C, gx = lay.g + 8 * C;       // gate table: this stage's, the next's, the last's
     int rec_phase = v.rec_stride > 0 ? (int)((step0 + 1) % v.rec_stride) : -1;
     const float4 c0 = F4(lay.sc);
-    StageCoef cf{c0.x, c0.y, c0.z};
+    StageCoef cf{c0.x, c0.y, c0.z, c0.w};
     float iext = 0.0f;
     long long rec_at = 0;
     // one stage; next: the index of the stage after it
@@ -272,7 +272,7 @@ __device__ __forceinline__ void dense_run(const NetView &v, const int b, const D
                 acc = ac;
                 V = ext_stage(y0, ylo, cf.cn, d);
             } else {
-                ext_step(y0, ylo, cf.fin, ac);
+                ext_step(y0, ylo, cf.fin, cf.finl, ac);
                 acc = 0.0f;
                 V = y0;
             }
@@ -282,7 +282,7 @@ __device__ __forceinline__ void dense_run(const NetView &v, const int b, const D
             }
         }
         const float4 c4 = F4(lay.sc + 16 * next);
-        cf = StageCoef{c4.x, c4.y, c4.z};
+        cf = StageCoef{c4.x, c4.y, c4.z, c4.w};
         __syncthreads();
         if (cl > 1) cluster_wait();
         int t = vc;

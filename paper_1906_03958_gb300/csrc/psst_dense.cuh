@@ -28,7 +28,7 @@ __device__ __forceinline__ void gate_update(const StageCoef &c, float al, float 
         st.z = ac;
         st.w = ext_stage(st.x, st.y, c.cn, d);
     } else {
-        ext_step(st.x, st.y, c.fin, ac);
+        ext_step(st.x, st.y, c.fin, c.finl, ac);
         st.z = 0.0f;
         st.w = st.x;
     }
@@ -49,7 +49,7 @@ __device__ __forceinline__ float pair_unit(const StageCoef &c, float a_, float b
         st.w = __fmul_rn(c.cn, kQ);
         return __fadd_rn(st.x, __fadd_rn(fmaf(st.w, st.x, st.z), st.y));
     }
-    ext_add(st.x, st.y, fmaf(__fmul_rn(c.fin, aQ), st.x, __fmul_rn(c.fin, aP)));
+    ext_add(st.x, st.y, fmaf(step_end(c, aQ), st.x, step_end(c, aP)));
     st.z = st.w = 0.0f;
     acc = make_float2(0.0f, 0.0f);
     return __fadd_rn(st.x, st.y);
@@ -85,8 +85,7 @@ __device__ __forceinline__ float pair_unit2(const StageCoef &c, const float *sp,
         q.w = __fmul_rn(c.cn, kX);
         s = __fadd_rn(q.x, __fadd_rn(fmaf(z.x, q.x, fmaf(q.w, r0, q.z)), q.y));
     } else {
-        ext_add(q.x, q.y, fmaf(__fmul_rn(c.fin, aZ), q.x,
-                               fmaf(__fmul_rn(c.fin, aX), r0, __fmul_rn(c.fin, aU))));
+        ext_add(q.x, q.y, fmaf(step_end(c, aZ), q.x, fmaf(step_end(c, aX), r0, step_end(c, aU))));
         q.z = q.w = 0.0f;
         z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         s = __fadd_rn(q.x, q.y);

@@ -298,6 +298,7 @@ extern "C" int psst_integrate_grid_noalloc(const psst_device_network *d, int64_t
     v.noise_thresh = d->noise_thresh;
     v.noise_amp = d->noise_amp;
     v.dt = d->dt;
+    psst::step_scale(v);
     v.state = d->state;
     v.rec = d->rec;
     v.rec_stride = d->rec_stride;

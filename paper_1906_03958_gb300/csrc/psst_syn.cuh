@@ -217,10 +217,12 @@ __host__ __device__ constexpr int tableau_stage(int n, int s) { return 4 * (n + 
 // Coefficients of stage ST: w, the weight of its slope in the step's sum
 // (relative to the first nonzero weight); cn = dt a_{s+1}, the factor of the
 // slope in the next stage's start; fin = dt times the scale of the sum at
-// the step's end.  RK4: w = 1, 2, 2, 1, cn = dt/2, dt/2, dt, fin = dt/6.
+// the step's end, finl its second part (step_scale).  RK4: w = 1, 2, 2, 1,
+// cn = dt/2, dt/2, dt, fin + finl = dt/6.
 struct StageCoef {
-    float w, cn, fin;
+    float w, cn, fin, finl;
 };
+
 
 template <int ST>
 __device__ __forceinline__ StageCoef stage_coef(const NetView &v, float dt) {
@@ -229,14 +231,17 @@ __device__ __forceinline__ StageCoef stage_coef(const NetView &v, float dt) {
         constexpr int s = ST & 3;
         c.w = v.rk_w[s];
         c.cn = s < 3 ? v.rk_c[s < 3 ? s : 0] * dt : 0.0f;
-        c.fin = v.rk_beta * dt;
     } else {
         c.w = (ST == 1 || ST == 2) ? 2.0f : 1.0f;
         c.cn = (ST == 2) ? dt : 0.5f * dt;
-        c.fin = ST == 4 ? dt : dt * (1.0f / 6.0f);
     }
+    c.fin = v.fin;
+    c.finl = v.finl;
     return c;
 }
+
+// A step's increment from the sum a of its weighted slopes.
+__device__ __forceinline__ float step_end(const StageCoef &c, float a) { return fmaf(c.fin, a, __fmul_rn(c.finl, a)); }
 
 // Stage descriptors: whether the stage is its step's first and last, its
 // coefficients, and the first stage's term of the step's sum.  StageCT<ST>
@@ -273,13 +278,13 @@ __device__ __forceinline__ StageRT stage_rt(const NetView &v, int s, float dt) {
     if (v.method == PSST_METHOD_TABLEAU) {
         r.c.w = v.rk_w[s];
         r.c.cn = s < 3 ? v.rk_c[s < 3 ? s : 0] * dt : 0.0f;
-        r.c.fin = v.rk_beta * dt;
     } else {
         const bool euler = v.method == PSST_METHOD_EULER;
         r.c.w = (!euler && (s == 1 || s == 2)) ? 2.0f : 1.0f;
         r.c.cn = (!euler && s == 2) ? dt : 0.5f * dt;
-        r.c.fin = euler ? dt : dt * (1.0f / 6.0f);
     }
+    r.c.fin = v.fin;
+    r.c.finl = v.finl;
     return r;
 }
 
@@ -551,7 +556,7 @@ template <bool HAS2, class SG>
 __device__ __forceinline__ void coef_update(const float *sp, float V, const SG &sg, float2 &cur, float2 &acc,
                                             float2 &fin, float4 &cur2, float4 &acc2, float4 &fin2) {
     const bool FIRST = sg.first, LAST = sg.last;
-    const float WGT = sg.c.w, cnext = sg.c.cn, dt6 = sg.c.fin;
+    const float WGT = sg.c.w, cnext = sg.c.cn;
     const float T = transmitter(V, sp);
     // explicit roundings: no product is contracted into an FMA or folded
     // with a constant stage weight, so every kernel and stage kind (constant
@@ -577,7 +582,7 @@ __device__ __forceinline__ void coef_update(const float *sp, float V, const SG &
         acc = A1;
         cur = make_float2(cnext * kP, cnext * kQ);
     } else {
-        fin = make_float2(dt6 * A1.x, dt6 * A1.y);
+        fin = make_float2(step_end(sg.c, A1.x), step_end(sg.c, A1.y));
     }
     if (HAS2) {
         const float K3 = sp[SP_K3], K4 = sp[SP_K4];
@@ -591,7 +596,7 @@ __device__ __forceinline__ void coef_update(const float *sp, float V, const SG &
             acc2 = A2;
             cur2 = make_float4(cnext * kU, cnext * kX, cnext * kZ, Kd);
         } else {
-            fin2 = make_float4(dt6 * A2.x, dt6 * A2.y, dt6 * A2.z, Kd);
+            fin2 = make_float4(step_end(sg.c, A2.x), step_end(sg.c, A2.y), step_end(sg.c, A2.z), Kd);
         }
     }
 }
@@ -658,7 +663,7 @@ template <class SG>
 __device__ __forceinline__ float neuron_v_post(const SG &sg, int i, const VPre &p, float isyn, float *y0,
                                               float *ylo, float *acc) {
     const bool FIRST = sg.first, LAST = sg.last;
-    const float WGT = sg.c.w, cnext = sg.c.cn, dt6 = sg.c.fin;
+    const float WGT = sg.c.w, cnext = sg.c.cn;
     const float d = __fmul_rn(__fsub_rn(p.ie, isyn), p.invC);
     const float ac = FIRST ? sg.first_term(d) : fmaf(WGT, d, p.acc);
     if (!LAST) {
@@ -666,7 +671,7 @@ __device__ __forceinline__ float neuron_v_post(const SG &sg, int i, const VPre &
         return ext_stage(p.y0, p.lo, cnext, d);
     }
     float hi = p.y0, lo = p.lo;
-    ext_step(hi, lo, dt6, ac);
+    ext_step(hi, lo, sg.c.fin, sg.c.finl, ac);
     y0[i] = hi;
     ylo[i] = lo;
     return hi;
@@ -684,7 +689,7 @@ template <class SG>
 __device__ __forceinline__ void neuron_gates(const SG &sg, int i, int n, float V, const float *ysc, float *ysn,
                                              float *y0, float *ylo, float *acc) {
     const bool FIRST = sg.first, LAST = sg.last;
-    const float WGT = sg.c.w, cnext = sg.c.cn, dt6 = sg.c.fin;
+    const float WGT = sg.c.w, cnext = sg.c.cn;
     const float m = ysc[i], h = ysc[n + i], nn = ysc[2 * n + i];
     const Rates q = hh_rates(V);
     float d[3];
@@ -701,7 +706,7 @@ __device__ __forceinline__ void neuron_gates(const SG &sg, int i, int n, float V
             yn = ext_stage(y0[ix], ylo[ix], cnext, d[x]);
         } else {
             float hi = y0[ix], lo = ylo[ix];
-            ext_step(hi, lo, dt6, ac);
+            ext_step(hi, lo, sg.c.fin, sg.c.finl, ac);
             y0[ix] = hi;
             ylo[ix] = lo;
             yn = hi;
