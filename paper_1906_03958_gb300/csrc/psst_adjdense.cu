@@ -24,8 +24,8 @@
 //      multiply-adds), the exchange among the eight threads, the pairs'
 //      adjoints; neuron warps, meanwhile: the gates' adjoints and the
 //      parameter gradients,
-// with one barrier after each.  Every 32 steps the gradients' partial sums go
-// to two-float totals.
+// with one barrier after each.  Every few steps the gradients' partial sums
+// go to two-float totals (FOLD_STEPS).
 //
 // Bound: the chain of a sweep stage (two barriers, sums, exchange) on 64
 // networks of 120 neurons, the recompute's stage on small ones.  It replaces,
@@ -48,7 +48,13 @@ namespace psst {
 
 namespace {
 
-constexpr int FOLD_STEPS = 32;
+// Steps whose weight-gradient terms run up in FP32 before they join the
+// two-float totals: at most a quarter of a segment (one rounding per stage and
+// at most four stages a step: no more than the one per step of a sum over the
+// whole segment, as psst_adjoint.cu forms it).  Weight gradients of 8 lobes,
+// 200 steps, from the float64 ones with 4 / 8 / 16 / 32 steps: 2.26 / 2.27 /
+// 2.31 / 2.46e-7; 64 lobes, forward and adjoint: 2741 / 2654 / 2619 / 2607 us.
+constexpr int FOLD_STEPS = 8;
 
 __device__ __forceinline__ unsigned cluster_rank() {
     unsigned r;
@@ -370,6 +376,7 @@ __device__ void sweep_run(const NetView &v, const AdjDenseView &av, const AdjDen
 
     const int SF = adj_stage_floats(N, Mp), step_bytes = 4 * ns * SF, nvec = ns * SF / 4, zb = 128 * Q * nt;
     const int ckpt = av.ckpt_every, nseg = (nsteps + ckpt - 1) / ckpt;
+    const int fold_steps = max(1, min(FOLD_STEPS, min(ckpt, nsteps) / 4));
     if (tid < TP) {
         // ---- pair warps: the sums over each slot's neurons, the pairs'
         // adjoints; the gradients' multiply-adds while the neuron warps
@@ -463,7 +470,7 @@ __device__ void sweep_run(const NetView &v, const AdjDenseView &av, const AdjDen
                     }
                     zc = zb - zc;
                 }
-                if (++since == FOLD_STEPS) {
+                if (++since == fold_steps) {
                     fold();
                     since = 0;
                 }
