@@ -121,8 +121,9 @@ typedef struct {
     int32_t item_chunks;           /* 4-synapse chunks per work item of the synaptic sum (1..64), 0 = tuned.
                                       CTA mode with block_threads and item_chunks both 0 holds the synapses of
                                       per-pair networks (gate_mode) as dense rows instead of work items where
-                                      they fit and no row has two synapses of one (presynaptic neuron, type)
-                                      pair; the two agree to rounding */
+                                      no row has two synapses of one (presynaptic neuron, type) pair, they fit
+                                      and the step is expected to be shorter so (by the networks' sizes,
+                                      connectivity and number); the two agree to rounding */
     int32_t device;                /* CUDA device ordinal, -1 = current device */
     int32_t gate_mode;             /* 0: one gate per (presynaptic neuron, type) pair whenever all
                                       its synapses' gates are equal (bitwise-identical results,

@@ -8,7 +8,9 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <map>
+#include <queue>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -454,7 +456,7 @@ int ctas_per_sm(const SmemCaps &caps, long long need) {
 // Smallest cluster size (1, 2, 4) whose CTAs all fit; 0 if none.  Per-pair
 // gates: the gate table gets the most copies (up to 32) that leave the CTAs
 // per SM as they are with one copy.
-int plan_network(const PlanInput &in, int b, const SmemCaps &caps, psst::NetPlan *pl, long long *need) {
+int plan_network(const PlanInput &in, int b, int min_cl, const SmemCaps &caps, psst::NetPlan *pl, long long *need) {
     const int n0 = in.net_off[b], N = in.net_off[b + 1] - n0, nt = in.nt;
     const bool has2 = in.flags[b] & psst::NET_HAS2, pair = in.flags[b] & psst::NET_PAIR;
     const std::vector<int> &n1 = in.n1, &n2 = in.n2;
@@ -462,13 +464,13 @@ int plan_network(const PlanInput &in, int b, const SmemCaps &caps, psst::NetPlan
     // a network spread over a larger cluster than it needs keeps the work-item
     // size of one CTA, so the summation order (and every result) is the same
     int user_K = in.user_K;
-    if (in.min_cl > 1 && N >= 2 * in.min_cl && user_K == 0) {
+    if (min_cl > 1 && N >= 2 * min_cl && user_K == 0) {
         std::vector<Share> sh1;
         make_shares(n1.data() + n0, n2.data() + n0, tc, nt, N, 1, 0, sh1, &user_K);
     }
     for (int cl = 1; cl <= PSST_MAX_CL; cl *= 2) {
         if (cl > 1 && N < 2 * cl) break;
-        if (cl < in.min_cl && N >= 2 * in.min_cl) continue;  // spread over a larger cluster
+        if (cl < min_cl && N >= 2 * min_cl) continue;  // spread over a larger cluster
         std::vector<Share> sh;
         int K = 1;
         make_shares(n1.data() + n0, n2.data() + n0, tc, nt, N, cl, user_K, sh, &K);
@@ -605,6 +607,122 @@ int plan_dense(const PlanInput &in, int b, int min_cl, bool alone, const SmemCap
         }
     }
     return 0;
+}
+
+// ---- dense rows or work items
+//
+// Dense rows cost the same whatever the connectivity, work items pay per chunk
+// of four synapses.  Times per RK4 step in us, fitted to networks of 20 to 500
+// neurons with two synapse types at 0.5 to 50% connectivity, 1 to 608 of them
+// (within a tenth for most; the table is in the design notes):
+//   an SM's time, when CTAs wait for SMs: items 0.58 + 0.0087 N + 0.00126 chunks,
+//     4.5 more on 2 CTAs and 9 on 4; dense rows 0.5 + 0.0037 N quads, 1.2 times
+//     that for the quads on 4 CTAs;
+//   alone on its SMs: items 2.6 + 0.0085 N + 0.0009 chunks / CTAs; dense rows
+//     1.5 + 0.0031 N quads / CTAs, 0.5 more on a cluster.
+// (Without the choice, dense rows wherever they fit: 304 networks of 300 neurons
+// at 1% 24.6 us against 7.6 with items, at 10% 24.9 against 14.0, of 400 at 5%
+// 53 against 16; 304 of 200 at 30% 11.7 against 13.2, one of 300 at 10% 4.3
+// against 7.1.)
+double item_cost(int N, double chunks, int cl, bool alone) {
+    return alone ? 2.6 + 0.0085 * N + 0.0009 * chunks / cl
+                 : 0.58 + 0.0087 * N + 0.00126 * chunks + (cl == 1 ? 0.0 : cl == 2 ? 4.5 : 9.0);
+}
+double dense_cost(int N, int nq, int cl, bool alone) {
+    return alone ? 1.5 + 0.0031 * N * nq / cl + (cl > 1 ? 0.5 : 0.0) : 0.5 + 0.0037 * N * nq * (cl == 4 ? 1.2 : 1.0);
+}
+
+// Time of a step of networks given as (SM time, time alone, CTAs): the longest
+// alone, or the fullest SM when each CTA goes to the least loaded one, the
+// largest first.
+struct NetCost {
+    double sm, alone;
+    int cl;
+};
+double step_time(const std::vector<NetCost> &nets, int sms) {
+    std::vector<double> ctas;
+    double t = 0.0;
+    for (const NetCost &c : nets) {
+        t = std::max(t, c.alone);
+        ctas.insert(ctas.end(), (size_t)c.cl, c.sm / c.cl);
+    }
+    std::sort(ctas.begin(), ctas.end(), std::greater<double>());
+    std::priority_queue<double, std::vector<double>, std::greater<double>> load;
+    for (int q = 0; q < sms; ++q) load.push(0.0);
+    for (double c : ctas) {
+        const double l = load.top() + c;
+        load.pop();
+        load.push(l);
+        t = std::max(t, l);
+    }
+    return t;
+}
+
+// Which networks take dense rows: those that can (plan_dense) and that run
+// faster so.  With SMs for all CTAs that is each network's time alone, with
+// clusters as large as there are SMs for.  With more CTAs it is the SM time each
+// takes, or for up to four times as many also the time alone, whichever gives
+// the shorter step (257 networks of 20 to 150 neurons, Euler, 300 steps: by SM
+// time 773 us, by time alone 677).  The choice sets the order of a row's sum, so
+// it does not depend on min_cluster or the autotuner's trials.
+std::vector<uint8_t> choose_dense(const PlanInput &in, const SmemCaps &caps, int sms) {
+    const int n_nets = in.n_nets, nt = in.nt;
+    std::vector<int> nets;  // networks that can take either
+    std::vector<double> chunks;
+    std::vector<int> icl, quads;
+    std::vector<NetCost> rest;  // the others with synapses
+    for (int b = 0; b < n_nets; ++b) {
+        if (in.net_syn[b] == 0) continue;
+        const int N = in.net_off[b + 1] - in.net_off[b];
+        psst::NetPlan pl;
+        psst::DensePlan dp;
+        long long need = 0;
+        int qr = 0;
+        double ch = 0.0;
+        for (int i = in.net_off[b]; i < in.net_off[b + 1]; ++i)
+            for (int t = 0; t < nt; ++t) ch += (in.tcnt[(size_t)i * nt + t] + 3) / 4;
+        const int cl = std::max(1, plan_network(in, b, 1, caps, &pl, &need));
+        if (need && plan_dense(in, b, 1, false, caps, &dp, &qr)) {
+            nets.push_back(b);
+            icl.push_back(cl);
+            quads.push_back(dp.nq);
+            chunks.push_back(ch);
+        } else {
+            rest.push_back({item_cost(N, ch, cl, false), item_cost(N, ch, cl, true), cl});
+        }
+    }
+    std::vector<uint8_t> dense((size_t)n_nets, 0);
+    // the choice by time alone on clusters of at least f CTAs, or by SM time
+    auto choose = [&](int f, bool alone, std::vector<uint8_t> &pick, std::vector<NetCost> &cost) {
+        pick.assign(nets.size(), 0);
+        cost = rest;
+        long long ctas = 0;
+        for (const NetCost &c : rest) ctas += c.cl;
+        for (size_t k = 0; k < nets.size(); ++k) {
+            const int b = nets[k], N = in.net_off[b + 1] - in.net_off[b];
+            psst::DensePlan dp;
+            int qr = 0;
+            const int dcl = plan_dense(in, b, f, alone, caps, &dp, &qr);
+            const NetCost d{dense_cost(N, quads[k], dcl, false), dense_cost(N, quads[k], dcl, true), dcl};
+            const NetCost i{item_cost(N, chunks[k], icl[k], false), item_cost(N, chunks[k], icl[k], true), icl[k]};
+            pick[k] = dcl && (alone ? d.alone <= 1.05 * i.alone : d.sm <= 1.05 * i.sm);
+            cost.push_back(pick[k] ? d : i);
+            ctas += cost.back().cl;
+        }
+        return ctas;
+    };
+    std::vector<uint8_t> pick, by_alone;
+    std::vector<NetCost> cost;
+    bool done = nets.empty();
+    for (int f = PSST_MAX_CL; !done && f >= 1 && (long long)nets.size() <= sms; f /= 2)
+        done = choose(f, true, pick, cost) <= sms;
+    if (!done && choose(1, false, pick, cost) <= 4LL * sms) {
+        const double by_sm = step_time(cost, sms);
+        choose(1, true, by_alone, cost);
+        if (step_time(cost, sms) < by_sm) pick = by_alone;
+    }
+    for (size_t k = 0; k < nets.size(); ++k) dense[nets[k]] = pick[k];
+    return dense;
 }
 
 // Threads that give every neuron's and every pair's unit one of its own
@@ -813,6 +931,10 @@ int setup_cta(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
     std::vector<psst::DensePlan> dplans((size_t)n_nets);
     std::vector<int> qr_of((size_t)n_nets, 0);
     std::vector<int> ind_neuron, ind_net;  // neurons of the networks without synapses
+    int sms = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    if (e != cudaSuccess) return *err = e, cuda_fail(e, "device attributes");
+    const std::vector<uint8_t> dense = choose_dense(in, caps, sms);
     for (int b = 0; b < n_nets; ++b) {
         const int n0 = in.net_off[b], N = in.net_off[b + 1] - n0;
         if (in.net_syn[b] == 0) {  // independent neurons: no size class, no barrier
@@ -825,12 +947,9 @@ int setup_cta(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
         }
         if ((long long)N * nt >= 65536)
             return fail(PSST_ERR_UNSUPPORTED, "net %d: %d neurons x %d synapse types must stay below 65536", b, N, nt);
-        // what CTA mode accepts is what the item kernel can hold; the dense
-        // kernel then takes the networks that it can (half the item kernel's
-        // time or less per network up to 120 neurons and where SMs are idle,
-        // 0.5 to 0.85 of it above, at 10 to 50% connectivity)
-        int cl = plan_network(in, b, caps, &plans[b], &need[b]);
-        const int dcl = cl ? plan_dense(in, b, in.min_cl, false, caps, &dplans[b], &qr_of[b]) : 0;
+        // what CTA mode accepts is what the item kernel can hold
+        int cl = plan_network(in, b, in.min_cl, caps, &plans[b], &need[b]);
+        const int dcl = cl && dense[b] ? plan_dense(in, b, in.min_cl, false, caps, &dplans[b], &qr_of[b]) : 0;
         if (dcl) {
             cl = dcl;
             plans[b].K = 0;
@@ -849,9 +968,6 @@ int setup_cta(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
     // clusters of twice as many CTAs, the costliest first (240 neurons alone:
     // 6.7 us per step on one CTA, 4.6 on two, 3.9 on four; results do not
     // depend on it)
-    int sms = 0;
-    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-    if (e != cudaSuccess) return *err = e, cuda_fail(e, "device attributes");
     long long ctas = 0;
     for (int b = 0; b < n_nets; ++b) ctas += cl_of[b];
     if (ctas <= sms)  // every CTA has an SM of its own
@@ -1069,7 +1185,7 @@ int psst_create_network(const psst_network_desc *d, const psst_allocator *a, pss
         if (pin.net_syn[b] == 0) continue;  // independent neurons need no shared-memory plan
         psst::NetPlan pl;
         long long need = 0;
-        all_fit = plan_network(pin, b, caps, &pl, &need) != 0;
+        all_fit = plan_network(pin, b, pin.min_cl, caps, &pl, &need) != 0;
     }
     int mode = d->mode;
     if (mode == PSST_MODE_AUTO) mode = all_fit ? PSST_MODE_CTA : PSST_MODE_GRID;
