@@ -87,6 +87,10 @@ struct psst_net {
     std::vector<psst::ClassLaunch> classes;  // CTA mode: one launch per size class
     std::vector<std::vector<int>> class_nets;  // the networks of each
     std::vector<psst::DensePlan> dplans;       // plans of the networks in dense classes
+    int *d_list = nullptr;                     // their device copies: launch lists and plans
+    psst::NetPlan *d_plans = nullptr;
+    psst::DensePlan *d_dplans = nullptr;
+    bool planned = false;                      // the launch plan is complete and fits the state's gates
     std::vector<void *> allocs;
     long long step = 0;       // global step index of the current state
     long long rec_reset = 0;  // step at which the record ring was last reset
@@ -1050,17 +1054,18 @@ int setup_cta(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
             h->classes.push_back(c);
         }
     }
-    int *dl = nullptr;
-    psst::NetPlan *dp = nullptr;
-    psst::DensePlan *ddp = nullptr;
-    e = upload(h, &dl, all_lists.data(), all_lists.size());
-    if (e == cudaSuccess) e = upload(h, &dp, plans.data(), plans.size());
-    if (e == cudaSuccess) e = upload(h, &ddp, dplans.data(), dplans.size());
+    // (the caller has waited for what used the present plan: replan)
+    h->drop(h->d_list);
+    h->drop(h->d_plans);
+    h->drop(h->d_dplans);
+    e = upload(h, &h->d_list, all_lists.data(), all_lists.size());
+    if (e == cudaSuccess) e = upload(h, &h->d_plans, plans.data(), plans.size());
+    if (e == cudaSuccess) e = upload(h, &h->d_dplans, dplans.data(), dplans.size());
     if (e == cudaSuccess) e = upload_columns(h, dplans, qr_of);
     for (size_t i = 0; e == cudaSuccess && i < h->classes.size(); ++i) {
-        h->classes[i].list = dl + ranges[i].first;
-        h->classes[i].plans = dp;
-        h->classes[i].dplans = ddp;
+        h->classes[i].list = h->d_list + ranges[i].first;
+        h->classes[i].plans = h->d_plans;
+        h->classes[i].dplans = h->d_dplans;
         if (h->classes[i].qr) {
             e = psst::dense_prepare(h->classes[i].qr, caps.max_dyn);
         } else {
@@ -1093,6 +1098,18 @@ int setup_cta(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
         else h->n_global += c.n_nets;
     }
     return PSST_OK;
+}
+
+// A new launch plan for the state's present gates and cluster sizes.  It
+// replaces buffers that launches still queued on st read, so it waits for them
+// first.  Until it succeeds the handle has no plan (launch_steps refuses).
+int replan(psst_net *h, cudaStream_t st, cudaError_t *err) {
+    h->planned = false;
+    const cudaError_t e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return *err = e, cuda_fail(e, "launch plan");
+    const int rc = h->mode == PSST_MODE_GRID ? setup_grid(h, h->caps, err) : setup_cta(h, h->caps, err);
+    h->planned = rc == PSST_OK;
+    return rc;
 }
 
 }  // namespace
@@ -1319,6 +1336,7 @@ int psst_create_network(const psst_network_desc *d, const psst_allocator *a, pss
         delete h;
         return rc;
     }
+    h->planned = true;
     *out = h;
     return PSST_OK;
 }
@@ -1333,6 +1351,8 @@ cudaError_t class_launch(const NetView &v, const psst::ClassLaunch &c, long long
 
 // Launch the kernels for n_steps steps starting at global step `step0`.
 int launch_steps(psst_net *h, long long step0, long long n_steps, cudaStream_t st) {
+    if (!h->planned)
+        return fail(PSST_ERR_STATE, "no launch plan: the last psst_set_state or psst_autotune could not make one");
     const long long chunk = 1LL << 30;
     const bool fork = h->mode != PSST_MODE_GRID && !h->class_streams.empty();
     if (fork) {
@@ -1456,32 +1476,41 @@ int replay_steps(psst_net *h, long long step0, long long n_steps, cudaStream_t s
 // every (presynaptic neuron, type) pair?  When that changes, the CTA-mode
 // plan (per-pair or per-synapse layout) is rebuilt.
 int recheck_pairs(psst_net *h, cudaStream_t st) {
-    if (h->pin.force_synapse_gates) return PSST_OK;
-    const int n_nets = h->pin.n_nets;
-    if (!h->d_check) {
-        cudaError_t e = h->alloc(&h->d_check, (size_t)n_nets);
-        if (e != cudaSuccess) return cuda_fail(e, "pair check buffer");
-    }
-    int max_m = 0;
-    for (int b = 0; b < n_nets; ++b) max_m = std::max(max_m, (h->pin.net_off[b + 1] - h->pin.net_off[b]) * h->pin.nt);
-    std::vector<uint8_t> ok((size_t)n_nets, 0);
-    if (4LL * max_m <= 200 * 1024) {
-        cudaError_t e = psst::pair_check(h->v, h->d_check, 4 * max_m, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(ok.data(), h->d_check, (size_t)n_nets, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return cuda_fail(e, "pair check");
-    }
+    const bool had_plan = h->planned;
+    h->planned = false;  // until the new state's gates are known to fit it
     bool changed = false;
-    for (int b = 0; b < n_nets; ++b) {
-        const uint8_t f = (uint8_t)((h->pin.flags[b] & psst::NET_HAS2) | (ok[b] ? psst::NET_PAIR : 0));
-        changed |= f != h->pin.flags[b];
-        h->pin.flags[b] = f;
+    cudaError_t e = cudaSuccess;
+    if (!h->pin.force_synapse_gates) {
+        const int n_nets = h->pin.n_nets;
+        if (!h->d_check) e = h->alloc(&h->d_check, (size_t)n_nets);
+        if (e != cudaSuccess) return cuda_fail(e, "pair check buffer");
+        int max_m = 0;
+        for (int b = 0; b < n_nets; ++b)
+            max_m = std::max(max_m, (h->pin.net_off[b + 1] - h->pin.net_off[b]) * h->pin.nt);
+        std::vector<uint8_t> ok((size_t)n_nets, 0);
+        if (4LL * max_m <= 200 * 1024) {
+            e = psst::pair_check(h->v, h->d_check, 4 * max_m, st);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(ok.data(), h->d_check, (size_t)n_nets, cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            if (e != cudaSuccess) return cuda_fail(e, "pair check");
+        }
+        for (int b = 0; b < n_nets; ++b) {
+            const uint8_t f = (uint8_t)((h->pin.flags[b] & psst::NET_HAS2) | (ok[b] ? psst::NET_PAIR : 0));
+            changed |= f != h->pin.flags[b];
+            h->pin.flags[b] = f;
+        }
     }
-    if (!changed) return PSST_OK;
-    cudaError_t e = cudaMemcpy((void *)h->v.net_flags, h->pin.flags.data(), (size_t)n_nets, cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_fail(e, "flags");
+    if (!changed && had_plan) {
+        h->planned = true;
+        return PSST_OK;
+    }
     h->drop_graph();
-    return h->mode == PSST_MODE_GRID ? setup_grid(h, h->caps, &e) : setup_cta(h, h->caps, &e);
+    e = cudaStreamSynchronize(st);  // launches still queued read the flags
+    if (e == cudaSuccess)
+        e = cudaMemcpy((void *)h->v.net_flags, h->pin.flags.data(), h->pin.flags.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return cuda_fail(e, "flags");
+    return replan(h, st, &e);
 }
 
 }  // namespace
@@ -1498,6 +1527,7 @@ int psst_autotune(psst_net *h, int64_t trial_steps, void *stream) {
     if (!h) return fail(PSST_ERR_INVALID_ARG, "handle is NULL");
     if (trial_steps < 1) return fail(PSST_ERR_INVALID_ARG, "trial_steps must be >= 1");
     if (h->mode != PSST_MODE_CTA) return PSST_OK;  // grid mode has one shape per device
+    if (!h->planned) return fail(PSST_ERR_STATE, "no launch plan: the last psst_set_state could not make one");
     DeviceGuard guard(h->device);
     cudaStream_t st = (cudaStream_t)stream;
     const size_t dim = (size_t)(4 * h->v.N + 2 * h->v.S);
@@ -1522,7 +1552,7 @@ int psst_autotune(psst_net *h, int64_t trial_steps, void *stream) {
         int best_cl = h->pin.min_cl;
         for (int mc = 1; mc <= PSST_MAX_CL && e == cudaSuccess; mc *= 2) {
             h->pin.min_cl = mc;
-            if (setup_cta(h, h->caps, &e) != PSST_OK) {
+            if (replan(h, st, &e) != PSST_OK) {
                 e = cudaSuccess;
                 continue;
             }
@@ -1541,7 +1571,7 @@ int psst_autotune(psst_net *h, int64_t trial_steps, void *stream) {
             }
         }
         h->pin.min_cl = best_cl;
-        if (e == cudaSuccess && setup_cta(h, h->caps, &e) != PSST_OK && e == cudaSuccess) e = cudaErrorUnknown;
+        if (e == cudaSuccess && replan(h, st, &e) != PSST_OK && e == cudaSuccess) e = cudaErrorUnknown;
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(h->v.state, h->tune_buf, dim * sizeof(float), cudaMemcpyDeviceToDevice, st);
     }
