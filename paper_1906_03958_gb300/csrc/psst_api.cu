@@ -1853,6 +1853,23 @@ int psst_set_neuron_params(psst_net *h, const float *p, size_t n, int on_device,
     return e == cudaSuccess ? PSST_OK : cuda_fail(e, "psst_set_neuron_params");
 }
 
+// Give back what the adjoint over work items alone uses.
+static void drop_adj_items(psst_net *h) {
+    h->adj_K.clear();
+    h->drop(h->d_adjK);
+    h->drop(h->d_adjI);
+    h->drop(h->d_adjKC);
+    h->drop(h->d_adjCI);
+    h->drop(h->d_cib);
+    h->drop(h->d_ciboff);
+    h->drop(h->d_ck);
+    h->drop(h->d_crow);
+    h->drop(h->d_cslotoff);
+    h->drop(h->adj_gpart);
+    h->drop(h->adj_gtot);
+    h->drop(h->d_segoff);
+}
+
 // Give back what the adjoint over dense rows alone uses.
 static void drop_adj_dense(psst_net *h) {
     h->drop(h->d_adjd_plans);
@@ -1940,10 +1957,12 @@ static int plan_adj_dense(psst_net *h) {
 // Segment buffers of at least `floats` floats.  On failure the present ones
 // stay, with the plans laid out for them; on success they stay allocated too
 // (an earlier call's kernel may still use them).
-static cudaError_t grow_segments(psst_net *h, long long floats) {
+static cudaError_t grow_segments(psst_net *h, long long floats, cudaStream_t st) {
     if (floats <= h->adj_seg_cap) return cudaSuccess;
     float *seg = nullptr;
-    const cudaError_t e = h->alloc(&seg, (size_t)floats);
+    cudaError_t e = h->alloc(&seg, (size_t)floats);
+    // (padding slots' records are copied, though never written or used)
+    if (e == cudaSuccess) e = cudaMemsetAsync(seg, 0, (size_t)floats * sizeof(float), st);
     if (e != cudaSuccess) return e;
     h->adj_seg = seg;
     h->adj_seg_cap = floats;
@@ -1962,7 +1981,7 @@ static int adjoint_dense(psst_net *h, long long s0, int n_steps, int ckpt_every,
             p.seg_off = total;
             total += 2 * span * ns * psst::adj_stage_floats(h->pin.net_off[b + 1] - h->pin.net_off[b], p.Mp);
         }
-        cudaError_t e = grow_segments(h, total);
+        cudaError_t e = grow_segments(h, total, st);
         if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint storage");
         h->adjd_span = -1;  // until the plans for it are there
         e = cudaMemcpyAsync(h->d_adjd_plans, h->adjd_plans.data(), h->adjd_plans.size() * sizeof(psst::AdjDensePlan),
@@ -1993,65 +2012,12 @@ static int adjoint_dense(psst_net *h, long long s0, int n_steps, int ckpt_every,
     return PSST_OK;
 }
 
-int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_frames, int32_t ckpt_every,
-                 float *grad_w, float *grad_neuron_params, float *grad_state0, void *stream) {
-    if (!h || !grad_w || !grad_neuron_params) return fail(PSST_ERR_INVALID_ARG, "NULL argument");
-    if (h->mode != PSST_MODE_CTA) return fail(PSST_ERR_UNSUPPORTED, "the adjoint runs in CTA mode only");
-    if (n_steps < 1 || n_steps > (1LL << 30)) return fail(PSST_ERR_INVALID_ARG, "n_steps must be in 1..2^30");
-    if (ckpt_every == 0) {
-        if (!h->rec_ck_valid || h->rec_ck_nsteps != n_steps)
-            return fail(PSST_ERR_STATE, "no checkpoints of a %lld-step integrate call are recorded", (long long)n_steps);
-    } else if (ckpt_every < 1) {
-        return fail(PSST_ERR_INVALID_ARG, "ckpt_every must be >= 1 (0 = recorded)");
-    }
-    const long long stride = h->v.rec_stride, s0 = ckpt_every == 0 ? h->rec_ck_start : h->step;
-    long long want = 0;
-    if (stride > 0) want = (s0 + n_steps) / stride - s0 / stride;
-    if (n_frames != want)
-        return fail(PSST_ERR_INVALID_ARG, "dL_dV has %lld frames, the span records %lld", (long long)n_frames, want);
-    if (n_frames > 0 && !dL_dV) return fail(PSST_ERR_INVALID_ARG, "dL_dV is NULL");
-    DeviceGuard guard(h->device);
+// The adjoint over work items (psst_adjoint.cu) of the recorded span.
+static int adjoint_items(psst_net *h, long long s0, long long n_steps, int ckpt_every, const float *dL_dV,
+                         long long n_frames, float *grad_w, float *grad_neuron_params, float *grad_state0,
+                         void *stream) {
     const int n_nets = h->v.n_nets, nt = h->v.n_stypes;
     cudaError_t e = cudaSuccess;
-    if (ckpt_every > 0) {
-        // The span's checkpoints: the forward kernel integrates it once from
-        // the current state, recording the state and its remainders every
-        // ckpt_every steps, so that each segment the adjoint recomputes
-        // starts on the forward kernel's trajectory; the network's state,
-        // step, record ring and recording setting are then put back.
-        const size_t dim = (size_t)(4 * h->v.N + 2 * h->v.S);
-        cudaStream_t st = (cudaStream_t)stream;
-        if (!h->tune_buf) e = h->alloc(&h->tune_buf, 2 * dim);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(h->tune_buf, h->v.state, dim * sizeof(float), cudaMemcpyDeviceToDevice, st);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(h->tune_buf + dim, h->v.state_lo, dim * sizeof(float), cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint state copy");
-        const int keep_every = h->rec_ck_every, keep_stride = h->v.rec_stride;
-        const long long keep_step = h->step;
-        h->v.rec_stride = 0;
-        int rc = psst_record_checkpoints(h, ckpt_every, n_steps);
-        if (rc == PSST_OK) rc = integrate_async(h, n_steps, st);
-        h->v.rec_stride = keep_stride;
-        h->rec_ck_every = keep_every;
-        h->rec_ck_cap_steps = keep_every > 0 ? (h->rec_ck_cap / (long long)dim) * keep_every : 0;
-        h->step = keep_step;
-        e = cudaMemcpyAsync(h->v.state, h->tune_buf, dim * sizeof(float), cudaMemcpyDeviceToDevice, st);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(h->v.state_lo, h->tune_buf + dim, dim * sizeof(float), cudaMemcpyDeviceToDevice, st);
-        if (rc != PSST_OK) return rc;
-        if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint state copy");
-    }
-    ckpt_every = h->rec_ck_spacing;
-    // small networks with one gate per pair: the adjoint over dense rows
-    bool pairs = true;
-    for (uint8_t f : h->pin.flags) pairs = pairs && (f & psst::NET_PAIR);
-    if (pairs && h->adjd_state == 0) {
-        const int rc = plan_adj_dense(h);
-        if (rc) return rc;
-    }
-    if (pairs && h->adjd_state == 1)
-        return adjoint_dense(h, s0, (int)n_steps, ckpt_every, dL_dV, (int)n_frames, grad_w, grad_neuron_params,
-                             grad_state0, (cudaStream_t)stream);
     // per-network plan (host copy of the CSR offsets is not kept: read them back once)
     if (h->adj_K.empty()) {
         std::vector<int> off((size_t)n_nets + 1);
@@ -2143,18 +2109,7 @@ int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_fra
         if (e == cudaSuccess && !h->adj_gy0) e = h->alloc(&h->adj_gy0, (size_t)h->v.N * 4);
         if (e == cudaSuccess) e = h->alloc(&h->d_segoff, (size_t)n_nets);
         if (e != cudaSuccess) {
-            h->drop(h->d_adjK);
-            h->drop(h->d_adjI);
-            h->drop(h->d_adjKC);
-            h->drop(h->d_adjCI);
-            h->drop(h->d_cib);
-            h->drop(h->d_ciboff);
-            h->drop(h->d_ck);
-            h->drop(h->d_crow);
-            h->drop(h->d_cslotoff);
-            h->drop(h->adj_gpart);
-            h->drop(h->adj_gtot);
-            h->drop(h->d_segoff);
+            drop_adj_items(h);
             return cuda_fail(e, "psst_adjoint buffers");
         }
         h->adj_K = adj_K;  // planned: only now that every buffer is there
@@ -2173,7 +2128,7 @@ int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_fra
             seg_total += 2LL * std::min<long long>(ckpt_every, n_steps) * step_floats;  // two buffers
         }
         h->adjd_span = -1;  // the buffer's layout is this path's now
-        e = grow_segments(h, seg_total);
+        e = grow_segments(h, seg_total, (cudaStream_t)stream);
         if (e == cudaSuccess) e = cudaMemcpy(h->d_segoff, sg.data(), sg.size() * sizeof(long long), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint storage");
     }
@@ -2205,6 +2160,81 @@ int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_fra
     if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint launch");
     h->launches = 2;
     return PSST_OK;
+}
+
+int psst_adjoint(psst_net *h, int64_t n_steps, const float *dL_dV, int64_t n_frames, int32_t ckpt_every,
+                 float *grad_w, float *grad_neuron_params, float *grad_state0, void *stream) {
+    if (!h || !grad_w || !grad_neuron_params) return fail(PSST_ERR_INVALID_ARG, "NULL argument");
+    if (h->mode != PSST_MODE_CTA) return fail(PSST_ERR_UNSUPPORTED, "the adjoint runs in CTA mode only");
+    if (n_steps < 1 || n_steps > (1LL << 30)) return fail(PSST_ERR_INVALID_ARG, "n_steps must be in 1..2^30");
+    if (ckpt_every == 0) {
+        if (!h->rec_ck_valid || h->rec_ck_nsteps != n_steps)
+            return fail(PSST_ERR_STATE, "no checkpoints of a %lld-step integrate call are recorded", (long long)n_steps);
+    } else if (ckpt_every < 1) {
+        return fail(PSST_ERR_INVALID_ARG, "ckpt_every must be >= 1 (0 = recorded)");
+    }
+    const long long stride = h->v.rec_stride, s0 = ckpt_every == 0 ? h->rec_ck_start : h->step;
+    long long want = 0;
+    if (stride > 0) want = (s0 + n_steps) / stride - s0 / stride;
+    if (n_frames != want)
+        return fail(PSST_ERR_INVALID_ARG, "dL_dV has %lld frames, the span records %lld", (long long)n_frames, want);
+    if (n_frames > 0 && !dL_dV) return fail(PSST_ERR_INVALID_ARG, "dL_dV is NULL");
+    DeviceGuard guard(h->device);
+    cudaError_t e = cudaSuccess;
+    if (ckpt_every > 0) {
+        // The span's checkpoints: the forward kernel integrates it once from
+        // the current state, recording the state and its remainders every
+        // ckpt_every steps, so that each segment the adjoint recomputes
+        // starts on the forward kernel's trajectory; the network's state,
+        // step, record ring and recording setting are then put back.
+        const size_t dim = (size_t)(4 * h->v.N + 2 * h->v.S);
+        cudaStream_t st = (cudaStream_t)stream;
+        if (!h->tune_buf) e = h->alloc(&h->tune_buf, 2 * dim);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h->tune_buf, h->v.state, dim * sizeof(float), cudaMemcpyDeviceToDevice, st);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(h->tune_buf + dim, h->v.state_lo, dim * sizeof(float), cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint state copy");
+        const int keep_every = h->rec_ck_every, keep_stride = h->v.rec_stride;
+        const long long keep_step = h->step;
+        h->v.rec_stride = 0;
+        int rc = psst_record_checkpoints(h, ckpt_every, n_steps);
+        if (rc == PSST_OK) rc = integrate_async(h, n_steps, st);
+        h->v.rec_stride = keep_stride;
+        h->rec_ck_every = keep_every;
+        h->rec_ck_cap_steps = keep_every > 0 ? (h->rec_ck_cap / (long long)dim) * keep_every : 0;
+        h->step = keep_step;
+        e = cudaMemcpyAsync(h->v.state, h->tune_buf, dim * sizeof(float), cudaMemcpyDeviceToDevice, st);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(h->v.state_lo, h->tune_buf + dim, dim * sizeof(float), cudaMemcpyDeviceToDevice, st);
+        if (rc != PSST_OK) return rc;
+        if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint state copy");
+    }
+    ckpt_every = h->rec_ck_spacing;
+    // small networks with one gate per pair: the adjoint over dense rows
+    bool pairs = true;
+    for (uint8_t f : h->pin.flags) pairs = pairs && (f & psst::NET_PAIR);
+    if (pairs && h->adjd_state == 0) {
+        const int rc = plan_adj_dense(h);
+        if (rc && rc != PSST_ERR_OOM) return rc;
+    }
+    if (pairs && h->adjd_state == 1) {
+        int rc = adjoint_dense(h, s0, (int)n_steps, ckpt_every, dL_dV, (int)n_frames, grad_w, grad_neuron_params,
+                               grad_state0, (cudaStream_t)stream);
+        if (rc != PSST_ERR_OOM) return rc;
+        // its records do not fit (a stage's are 12 N + 4 slots floats, the others'
+        // 6 N + 3 per pair): the adjoint over work items for this span, if need be
+        // with what this one holds given back for good
+        rc = adjoint_items(h, s0, n_steps, ckpt_every, dL_dV, n_frames, grad_w, grad_neuron_params, grad_state0, stream);
+        if (rc != PSST_ERR_OOM) return rc;
+        e = cudaStreamSynchronize((cudaStream_t)stream);
+        if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint");
+        drop_adj_dense(h);
+        rc = adjoint_items(h, s0, n_steps, ckpt_every, dL_dV, n_frames, grad_w, grad_neuron_params, grad_state0, stream);
+        h->adjd_state = rc == PSST_OK ? -1 : 0;
+        if (rc != PSST_OK) drop_adj_items(h);  // a shorter span plans again (nothing was launched)
+        return rc;
+    }
+    return adjoint_items(h, s0, n_steps, ckpt_every, dL_dV, n_frames, grad_w, grad_neuron_params, grad_state0, stream);
 }
 
 int psst_query(const psst_net *h, psst_info *out) {

@@ -84,3 +84,38 @@ def test_adjoint_refused_twice():
             with pytest.raises(psst.PsstError) as e:
                 _adjoint(net, 40, 40)
             assert e.value.code == -7  # PSST_ERR_UNSUPPORTED
+
+
+def test_dense_adjoint_gives_way_at_a_memory_limit():
+    # one synapse type, where the dense rows' records are larger: a limit that the
+    # adjoint over work items just meets
+    from paper_1906_03958_gb300 import psst
+    rng = np.random.default_rng(8)
+    n = 128
+    post, pre = np.nonzero(rng.random((n, n)) < 0.1)
+    spec = ng.single_network(np.zeros(n), rng.uniform(0.0, 8.0, n), post, pre, rng.uniform(0.0, 0.05, post.size),
+                             np.zeros(post.size), ng.neuron_table(ng.HH), ng.synapse_table(ng.ACH))
+    steps = 200
+
+    def run(gate_mode, limit):
+        alloc = _limited_allocator()
+        with psst.Network(spec, rec_stride=10, rec_capacity=20, gate_mode=gate_mode, allocator=alloc) as net:
+            net.record_checkpoints(steps, steps)
+            net.autotune(1)
+            base = alloc.used()
+            if limit is not None:
+                alloc.limit = base + limit
+            out = _adjoint(net, steps, steps)
+            again = _adjoint(net, steps, steps)
+            for a, b in zip(out, again):
+                np.testing.assert_array_equal(a, b)
+            return out, alloc.used() - base
+
+    general, need = run(1, None)
+    dense, more = run(0, None)
+    assert more > need
+    got, used = run(0, need)
+    assert used <= need
+    for a, b, c in zip(got, general, dense):
+        scale = np.abs(c).max()
+        assert np.abs(a - c).max() <= 1e-4 * scale and np.abs(b - c).max() <= 1e-4 * scale
