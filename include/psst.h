@@ -192,8 +192,9 @@ int psst_create_network(const psst_network_desc *d, const psst_allocator *a, pss
    FP32 trajectory tracks the exact RK4 map far more closely than plain
    FP32 accumulation.  Asynchronous on `stream`;
    device-side failures (NONFINITE, TIMEOUT) are reported by psst_status
-   (once a network holds a NaN or infinity, the values of its other neurons
-   are unspecified; other networks of the batch are not affected).
+   (a neuron that became NaN or infinite takes along those its synapses
+   reach, and with work items or in grid mode possibly others of its
+   network; other networks of the batch are not affected).
    With the environment variable PSST_SYNC set (to anything but "0") the
    call synchronises `stream` and returns what psst_status would.
    n_steps = 0 is a no-op.  Errors: INVALID_ARG (n_steps < 0), CUDA. */

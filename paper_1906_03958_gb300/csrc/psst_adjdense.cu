@@ -189,7 +189,7 @@ struct Recompute {
                 F4(lay.pst2 + 32 * (p - pl.np1) + 16) = make_float4(0.f, 0.f, 0.f, 0.f);
                 g = second_gate(__fadd_rn(s, sl), stab[(info.y >> 24) * ST_COLS + SP_KD]);
             }
-            F1(lay.g + (info.y & 0xFFFFFF)) = g;
+            F1(lay.g + (info.y & 0xFFFFFF)) = bounded(g);
         }
         __syncthreads();
         const int SF = adj_stage_floats(N, pl.Mp);
@@ -211,7 +211,7 @@ struct Recompute {
                 const float bb = __fadd_rn(a_, sp[SP_B]), r = F1(gc + (info.y & 0xFFFFFF));  // G = r
                 *(float4 *)(rec + 12 * N + 4 * info.z) =
                     make_float4(bb, a_ * (1.0f - T) * (sp[SP_KP] * 0.693147181f) * (1.0f - r), 0.0f, r);
-                F1(gn + (info.y & 0xFFFFFF)) = pair_unit<LAST>(cf, a_, bb, st, a);
+                F1(gn + (info.y & 0xFFFFFF)) = bounded(pair_unit<LAST>(cf, a_, bb, st, a));
                 F4(lay.pst + 16 * p) = st;
                 *(float2 *)(dsm + lay.pacc + 8 * p) = a;
             }
@@ -233,7 +233,7 @@ struct Recompute {
                                 __fdiv_rn(4.0f * s2 * s * sp[SP_KD], den * den), F1(gc + (info.y & 0xFFFFFF)));
                 const float r0 = st.x, sP = st.z, sQ = st.w;
                 pair_unit<LAST>(cf, a_, bb, st, a);
-                F1(gn + (info.y & 0xFFFFFF)) = pair_unit2<LAST>(cf, sp, r0, sP, sQ, q, z);
+                F1(gn + (info.y & 0xFFFFFF)) = bounded(pair_unit2<LAST>(cf, sp, r0, sP, sQ, q, z));
                 F4(lay.pst + 16 * p) = st;
                 *(float2 *)(dsm + lay.pacc + 8 * p) = a;
                 F4(lay.pst2 + 32 * p2) = q;
@@ -563,7 +563,7 @@ __device__ void sweep_run(const NetView &v, const AdjDenseView &av, const AdjDen
                         const int z = lay.z + zc + 4 * i;
 #pragma unroll
                         for (int t = 0; t < 4; ++t)
-                            if (t < nt) F1(z + 128 * Q * t) = o.q * (V - E[t]);
+                            if (t < nt) F1(z + 128 * Q * t) = bounded(o.q * (V - E[t]));
                     }
                     bar_all();
 #pragma unroll

@@ -183,7 +183,7 @@ __device__ __forceinline__ void dense_run(const NetView &v, const int b, const D
             F4(lay.pst2 + 32 * (p - np1) + 16) = make_float4(0.f, 0.f, 0.f, 0.f);
             g = second_gate(__fadd_rn(s, sl), stab[t * ST_COLS + SP_KD]);
         }
-        put(lay.g + 4 * col, cl, g);
+        put(lay.g + 4 * col, cl, bounded(g));
     }
     __syncthreads();
     if (cl > 1) {
@@ -215,7 +215,7 @@ __device__ __forceinline__ void dense_run(const NetView &v, const int b, const D
             const int2 info = *(const int2 *)(dsm + lay.pinfo + 8 * p);
             float2 a = *(const float2 *)(dsm + lay.pacc + 8 * p);
             const float g = pair_unit<LAST>(cf, stab + (info.y >> 24) * ST_COLS, F1(vc + info.x), st, a);
-            put(gn + (info.y & 0xFFFFFF), cl, g);
+            put(gn + (info.y & 0xFFFFFF), cl, bounded(g));
             F4(lay.pst + 16 * p) = st;
             *(float2 *)(dsm + lay.pacc + 8 * p) = a;
         }
@@ -228,7 +228,7 @@ __device__ __forceinline__ void dense_run(const NetView &v, const int b, const D
             const float *sp = stab + (info.y >> 24) * ST_COLS;
             const float r0 = st.x, sP = st.z, sQ = st.w;
             pair_unit<LAST>(cf, sp, F1(vc + info.x), st, a);
-            put(gn + (info.y & 0xFFFFFF), cl, pair_unit2<LAST>(cf, sp, r0, sP, sQ, q, z));
+            put(gn + (info.y & 0xFFFFFF), cl, bounded(pair_unit2<LAST>(cf, sp, r0, sP, sQ, q, z)));
             F4(lay.pst + 16 * p) = st;
             *(float2 *)(dsm + lay.pacc + 8 * p) = a;
             F4(lay.pst2 + 32 * p2) = q;

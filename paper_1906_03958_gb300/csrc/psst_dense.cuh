@@ -121,6 +121,13 @@ __device__ __forceinline__ void quad(const float4 (&w)[4], float4 g, float E, co
     }
 }
 
+// The largest finite number in place of one that is not finite.  Absent synapses
+// are weights of 0: with such a gate in the table they add 0 to their rows and
+// not NaN, while a present synapse drives its neuron out as well.  (Two versions
+// of the sums, with and without absent synapses, made a stage 5 to 18% longer, a
+// look through the row's synapses 5 to 10%.)
+__device__ __forceinline__ float bounded(float x) { return fmaxf(fminf(x, 3.402823466e38f), -3.402823466e38f); }
+
 // Sum over the eight threads of a row group: thread l gets row
 // 2 (l & 1) + (l >> 1 & 1).
 __device__ __forceinline__ float row_sum(const float (&a)[4], int l) {
