@@ -126,8 +126,11 @@ typedef struct {
                                       connectivity and number); the two agree to rounding */
     int32_t device;                /* CUDA device ordinal, -1 = current device */
     int32_t gate_mode;             /* 0: one gate per (presynaptic neuron, type) pair whenever all
-                                      its synapses' gates are equal (bitwise-identical results,
-                                      less work), else one per synapse; 1: always one per synapse */
+                                      its synapses' gates are equal (less work), else one per
+                                      synapse; 1: always one per synapse.  The layouts run other
+                                      kernels, which sum a row's synapses in another order and
+                                      agree to rounding; psst_set_state with other gates can
+                                      change a network's layout */
     int32_t method;                /* PSST_METHOD_RK4 (0), PSST_METHOD_EULER (1) or PSST_METHOD_TABLEAU (2) */
     int32_t min_cluster;           /* CTA mode: spread every network of at least 2 x min_cluster neurons
                                       over a cluster of at least min_cluster CTAs (1, 2 or 4; same
@@ -159,6 +162,7 @@ typedef struct {
                                       when no valid recording exists (none made, or the state, step,
                                       weights or neuron table changed since) */
     int64_t ck_steps;              /* steps of that recorded call (0 when ck_start is -1) */
+    int32_t adjoint;               /* the last psst_adjoint ran over dense rows (1) or work items (2); 0: none yet */
 } psst_info;
 
 typedef struct psst_net psst_net;
@@ -300,6 +304,11 @@ int psst_record_checkpoints(psst_net *h, int32_t every, int64_t max_steps);
    ckpt_every = 0 differentiates instead the span of the last psst_integrate
    call, whose checkpoints were recorded (psst_record_checkpoints); n_steps
    must equal that call's; PSST_ERR_STATE if no such checkpoints exist.
+   Networks of at most 128 neurons, 4 synapse types and 160 pair slots (each
+   type's used (presynaptic neuron, type) pairs rounded up to 4), one gate per
+   pair and no two synapses of one pair in a row run over dense rows, when
+   every network of the handle is one; otherwise the whole handle takes the
+   adjoint over work items, at about a third of the speed (psst_info.adjoint).
    Preconditions: CTA mode (else PSST_ERR_UNSUPPORTED); every network fits one CTA for the adjoint; all
    gates of a (presynaptic neuron, synapse type) pair hold the same value at
    the start (true from rest), else the device reports PSST_ERR_UNSUPPORTED

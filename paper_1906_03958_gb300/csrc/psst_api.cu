@@ -122,6 +122,7 @@ struct psst_net {
     unsigned short *d_adjd_slot = nullptr, *d_adjd_col = nullptr;
     float2 *adjd_gtot = nullptr;
     int adj_ckpt_every = 0;
+    int adj_ran = 0;  // psst_info.adjoint
     // checkpoints recorded by psst_integrate for a later psst_adjoint
     int rec_ck_every = 0;
     int rec_ck_spacing = 0;  // checkpoint spacing of the valid recording
@@ -2009,6 +2010,7 @@ static int adjoint_dense(psst_net *h, long long s0, int n_steps, int ckpt_every,
                                                  h->n_ntypes, grad_np, st);
     if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint launch");
     h->launches = 2;
+    h->adj_ran = 1;
     return PSST_OK;
 }
 
@@ -2159,6 +2161,7 @@ static int adjoint_items(psst_net *h, long long s0, long long n_steps, int ckpt_
                          (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "psst_adjoint launch");
     h->launches = 2;
+    h->adj_ran = 2;
     return PSST_OK;
 }
 
@@ -2262,6 +2265,7 @@ int psst_query(const psst_net *h, psst_info *out) {
     }
     out->ck_start = h->rec_ck_valid ? h->rec_ck_start : -1;
     out->ck_steps = h->rec_ck_valid ? h->rec_ck_nsteps : 0;
+    out->adjoint = h->adj_ran;
     return PSST_OK;
 }
 

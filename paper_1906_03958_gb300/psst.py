@@ -73,7 +73,7 @@ class Info(C.Structure):
                 ("smem_bytes", C.c_int32), ("n_single_cta_nets", C.c_int32),
                 ("n_cluster_nets", C.c_int32), ("n_launch_classes", C.c_int32),
                 ("kernel_launches", C.c_int32), ("n_pair_gate_nets", C.c_int32),
-                ("n_independent_nets", C.c_int32), ("ck_start", C.c_int64), ("ck_steps", C.c_int64)]
+                ("n_independent_nets", C.c_int32), ("ck_start", C.c_int64), ("ck_steps", C.c_int64), ("adjoint", C.c_int32)]
 
 
 _lib = None
