@@ -123,7 +123,8 @@ def measured_peaks():
 # Sources that decide each kernel's memory traffic: its own file, the
 # shared device headers and the host planner (launch shapes, layouts).
 KERNEL_SOURCES = {
-    "dense_kernel": ("psst_dense.cu", "psst_dense.cuh", "psst_syn.cuh"),
+    # the batch's size classes: dense_kernel and net_kernel, as the planner has it
+    "batch_kernels": ("psst_dense.cu", "psst_dense.cuh", "psst_cta.cu", "psst_syn.cuh"),
     "net_kernel": ("psst_cta.cu", "psst_syn.cuh"),
     "grid_kernel": ("psst_grid.cu", "psst_syn.cuh"),
     "adj_dense_kernel": ("psst_adjdense.cu", "psst_dense.cuh", "psst_syn.cuh"),
@@ -558,8 +559,8 @@ def main():
     dur = t_local / args.steps
     roof = {"bound": "alu", "achieved": flops_call / dur / 1e12, "peak": peak_tflops, "unit": "TFLOP/s",
             "frac": flops_call / dur / 1e12 / peak_tflops,
-            "traffic": traffic_for("dense_kernel", args.workload),
-            "kernel": f"dense_kernel: the {info['n_launch_classes']} size-class launches of one integrate call",
+            "traffic": traffic_for("batch_kernels", args.workload),
+            "kernel": f"dense_kernel and net_kernel: the {info['n_launch_classes']} size-class launches of one integrate call",
             "gates": "per (presynaptic neuron, type) pair" if pair_gates else "per synapse",
             "peak_source": f"FP32 FMA pipes: {n_sms} SMs x {FP32_LANES_PER_SM} lanes x 2 x "
                            f"{smax:.0f} MHz (sm_max_mhz of MEASURED_PEAKS.json)"}

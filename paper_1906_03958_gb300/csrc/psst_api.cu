@@ -619,7 +619,7 @@ int plan_dense(const PlanInput &in, int b, int min_cl, bool alone, const SmemCap
 // Dense rows cost the same whatever the connectivity, work items pay per chunk
 // of four synapses.  Times per RK4 step in us, fitted to networks of 20 to 500
 // neurons with two synapse types at 0.5 to 50% connectivity, 1 to 608 of them
-// (within a tenth for most; the table is in the design notes):
+// (within a tenth for most):
 //   an SM's time, when CTAs wait for SMs: items 0.58 + 0.0087 N + 0.00126 chunks,
 //     4.5 more on 2 CTAs and 9 on 4; dense rows 0.5 + 0.0037 N quads, 1.2 times
 //     that for the quads on 4 CTAs;

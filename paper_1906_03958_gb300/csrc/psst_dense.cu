@@ -29,14 +29,17 @@
 // ahead in pushing is impossible, so the buffer it writes is never one still
 // read.
 //
-// Bound: instruction issue (62% of the slots with the 12 warps of a
-// 180-neuron CTA, 5,800 warp instructions a stage, 3,350 of them on the FMA
-// pipe, 26 per quad of 16 multiply-adds); alone on its SM, the chain of one
-// stage (rates, or sums, exchange and potential: about 500 cycles).  Measured
-// against the work-item kernel (psst_cta.cu), us per RK4 step, before / now:
-// antennal lobe 6.5 / 3.2, 300 neurons alone 17 / 4.1, 304 networks of 60
-// neurons 4.7 / 2.4, of 120 8.0 / 3.9, of 180 16.8 / 8.4, of 240 26.3 / 13.5,
-// of 300 34.2 / 23.6; 4,096 networks of 20 to 300 neurons 146 / 128.
+// Bound: instruction issue (60% of the slots with the 12 warps of a
+// 180-neuron CTA, 5,180 warp instructions a stage, 3,270 of them on the FMA
+// pipe; a quad of 16 multiply-adds is 26, 24 of them there and two loads);
+// alone on its SM, the chain of one stage (rates, or sums, exchange and
+// potential: about 500 cycles).  Measured against the work-item kernel
+// (psst_cta.cu), us per RK4 step, work items / dense rows: antennal lobe 6.5 /
+// 3.1; at 30% connectivity 300 neurons alone 7.9 / 4.3, 608 networks of 60
+// neurons 5.4 / 3.9, of 120 12.0 / 8.2, of 150 14.9 / 14.0, 304 of 180 10.9 /
+// 8.8, of 250 20.8 / 17.9, of 300 32.5 / 25.9.  Its cost does not fall with the
+// connectivity, the work items' does: the planner chooses (choose_dense in
+// psst_api.cu).
 #include <cuda_runtime.h>
 
 #include <type_traits>

@@ -25,7 +25,7 @@
 // at stage s only, so it is published at the start of stage s and travels
 // while that stage's table copy, sums and potentials run (published at the
 // stage's end, every stage waited for the slowest CTA's words: 10,000 neurons
-// 20.1 -> 15.6 us per step, 3,764 12.4 -> 10.1, 1,800 9.7 -> 9.1).
+// 17.8 -> 16.7 us per step, 3,764 12.4 -> 10.1, 1,800 9.7 -> 9.1).
 // Each CTA also writes one tagged heartbeat word per stage, after its own copy
 // of the stage's table.  Three tables, by phase modulo 3: the words of phase
 // q + 1 overwrite those of phase q - 2 by a CTA that has gathered phase q - 1,
