@@ -201,7 +201,9 @@ int psst_create_network(const psst_network_desc *d, const psst_allocator *a, pss
    network; other networks of the batch are not affected).
    With the environment variable PSST_SYNC set (to anything but "0") the
    call synchronises `stream` and returns what psst_status would.
-   n_steps = 0 is a no-op.  Errors: INVALID_ARG (n_steps < 0), CUDA. */
+   n_steps = 0 is a no-op.  Errors: INVALID_ARG (n_steps < 0), CUDA, STATE
+   (no launch plan: psst_set_state or psst_autotune failed to make one; a
+   psst_set_state that succeeds makes it). */
 int psst_integrate(psst_net *h, int64_t n_steps, void *stream);
 
 /* Grid mode only: time limit of one wait at the device-wide barrier between
