@@ -624,26 +624,33 @@ int plan_dense(const PlanInput &in, int b, int min_cl, bool alone, const SmemCap
 //     4.5 more on 2 CTAs and 9 on 4; dense rows 0.5 + 0.0037 N quads, 1.2 times
 //     that for the quads on 4 CTAs;
 //   alone on its SMs: items 2.6 + 0.0085 N + 0.0009 chunks / CTAs; dense rows
-//     1.5 + 0.0031 N quads / CTAs, 0.5 more on a cluster.
+//     1.5 + 0.0031 N quads / CTAs, 0.5 more on a cluster;
+//   once per call (taken as 100 steps): items 18 + 0.0042 synapses / CTAs, dense
+//     rows 17 + 0.0007 synapses / CTAs, alone.
 // (Without the choice, dense rows wherever they fit: 304 networks of 300 neurons
 // at 1% 24.6 us against 7.6 with items, at 10% 24.9 against 14.0, of 400 at 5%
 // 53 against 16; 304 of 200 at 30% 11.7 against 13.2, one of 300 at 10% 4.3
 // against 7.1.)
-double item_cost(int N, double chunks, int cl, bool alone) {
-    return alone ? 2.6 + 0.0085 * N + 0.0009 * chunks / cl
-                 : 0.58 + 0.0087 * N + 0.00126 * chunks + (cl == 1 ? 0.0 : cl == 2 ? 4.5 : 9.0);
+struct NetCost {
+    double sm, alone;  // us per step: an SM's time, alone on its SMs
+    int cl;
+};
+NetCost with_call(double sm, double alone, double call, int stages, int cl) {
+    const double per_step = call / 100.0;
+    return {sm * stages / 4 + per_step * sm / alone, alone * stages / 4 + per_step, cl};
 }
-double dense_cost(int N, int nq, int cl, bool alone) {
-    return alone ? 1.5 + 0.0031 * N * nq / cl + (cl > 1 ? 0.5 : 0.0) : 0.5 + 0.0037 * N * nq * (cl == 4 ? 1.2 : 1.0);
+NetCost item_cost(int N, double chunks, double syn, int cl, int stages) {
+    return with_call(0.58 + 0.0087 * N + 0.00126 * chunks + (cl == 1 ? 0.0 : cl == 2 ? 4.5 : 9.0),
+                     2.6 + 0.0085 * N + 0.0009 * chunks / cl, 18 + 0.0042 * syn / cl, stages, cl);
+}
+NetCost dense_cost(int N, int nq, double syn, int cl, int stages) {
+    return with_call(0.5 + 0.0037 * N * nq * (cl == 1 ? 1.0 : cl == 2 ? 1.1 : 1.2),
+                     1.5 + 0.0031 * N * nq / cl + (cl > 1 ? 0.5 : 0.0), 17 + 0.0007 * syn / cl, stages, cl);
 }
 
 // Time of a step of networks given as (SM time, time alone, CTAs): the longest
 // alone, or the fullest SM when each CTA goes to the least loaded one, the
-// largest first.
-struct NetCost {
-    double sm, alone;
-    int cl;
-};
+// largest first (so many CTAs that this evens out: the SM time over all SMs).
 double step_time(const std::vector<NetCost> &nets, int sms) {
     std::vector<double> ctas;
     double t = 0.0;
@@ -651,6 +658,7 @@ double step_time(const std::vector<NetCost> &nets, int sms) {
         t = std::max(t, c.alone);
         ctas.insert(ctas.end(), (size_t)c.cl, c.sm / c.cl);
     }
+    if (ctas.size() > 4 * (size_t)sms) return std::max(t, std::accumulate(ctas.begin(), ctas.end(), 0.0) / sms);
     std::sort(ctas.begin(), ctas.end(), std::greater<double>());
     std::priority_queue<double, std::vector<double>, std::greater<double>> load;
     for (int q = 0; q < sms; ++q) load.push(0.0);
@@ -663,19 +671,19 @@ double step_time(const std::vector<NetCost> &nets, int sms) {
     return t;
 }
 
-// Which networks take dense rows: those that can (plan_dense) and that run
-// faster so.  With SMs for all CTAs that is each network's time alone, with
-// clusters as large as there are SMs for.  With more CTAs it is the SM time each
-// takes, or for up to four times as many also the time alone, whichever gives
-// the shorter step (257 networks of 20 to 150 neurons, Euler, 300 steps: by SM
-// time 773 us, by time alone 677).  The choice sets the order of a row's sum, so
-// it does not depend on min_cluster or the autotuner's trials.
-std::vector<uint8_t> choose_dense(const PlanInput &in, const SmemCaps &caps, int sms) {
+// Which networks take dense rows, of those that can (plan_dense).  With SMs for
+// all CTAs: each that is not slower alone by a tenth, on clusters as large as
+// there are SMs for.  With more CTAs: all, unless giving work items to those
+// whose SM time (or time alone) is a seventh shorter with them makes the step
+// shorter by 6%; nearer ties were as often losses, from more size classes and
+// the work items' longer setup (400 networks of 10 to 200 neurons, Euler, 100
+// steps: 460 us with the nearest choice per network, 336 all dense; 257 of 20 to
+// 150, Euler, 300 steps: 773 and 677).  The choice sets the order of a row's
+// sum, so it does not depend on min_cluster or the autotuner's trials.
+std::vector<uint8_t> choose_dense(const PlanInput &in, const SmemCaps &caps, int sms, int stages) {
     const int n_nets = in.n_nets, nt = in.nt;
-    std::vector<int> nets;  // networks that can take either
-    std::vector<double> chunks;
-    std::vector<int> icl, quads;
-    std::vector<NetCost> rest;  // the others with synapses
+    std::vector<int> nets, quads;  // networks that can take either
+    std::vector<NetCost> items, rest;  // their costs with work items; the other networks with synapses
     for (int b = 0; b < n_nets; ++b) {
         if (in.net_syn[b] == 0) continue;
         const int N = in.net_off[b + 1] - in.net_off[b];
@@ -687,18 +695,18 @@ std::vector<uint8_t> choose_dense(const PlanInput &in, const SmemCaps &caps, int
         for (int i = in.net_off[b]; i < in.net_off[b + 1]; ++i)
             for (int t = 0; t < nt; ++t) ch += (in.tcnt[(size_t)i * nt + t] + 3) / 4;
         const int cl = std::max(1, plan_network(in, b, 1, caps, &pl, &need));
+        const NetCost c = item_cost(N, ch, (double)in.net_syn[b], cl, stages);
         if (need && plan_dense(in, b, 1, false, caps, &dp, &qr)) {
             nets.push_back(b);
-            icl.push_back(cl);
             quads.push_back(dp.nq);
-            chunks.push_back(ch);
+            items.push_back(c);
         } else {
-            rest.push_back({item_cost(N, ch, cl, false), item_cost(N, ch, cl, true), cl});
+            rest.push_back(c);
         }
     }
-    std::vector<uint8_t> dense((size_t)n_nets, 0);
-    // the choice by time alone on clusters of at least f CTAs, or by SM time
-    auto choose = [&](int f, bool alone, std::vector<uint8_t> &pick, std::vector<NetCost> &cost) {
+    // dense rows for network k on at least f CTAs where keep(dense, items)
+    std::vector<NetCost> cost;
+    auto choose = [&](int f, auto keep, std::vector<uint8_t> &pick) {
         pick.assign(nets.size(), 0);
         cost = rest;
         long long ctas = 0;
@@ -707,25 +715,33 @@ std::vector<uint8_t> choose_dense(const PlanInput &in, const SmemCaps &caps, int
             const int b = nets[k], N = in.net_off[b + 1] - in.net_off[b];
             psst::DensePlan dp;
             int qr = 0;
-            const int dcl = plan_dense(in, b, f, alone, caps, &dp, &qr);
-            const NetCost d{dense_cost(N, quads[k], dcl, false), dense_cost(N, quads[k], dcl, true), dcl};
-            const NetCost i{item_cost(N, chunks[k], icl[k], false), item_cost(N, chunks[k], icl[k], true), icl[k]};
-            pick[k] = dcl && (alone ? d.alone <= 1.05 * i.alone : d.sm <= 1.05 * i.sm);
-            cost.push_back(pick[k] ? d : i);
+            const int cl = plan_dense(in, b, f, f > 1, caps, &dp, &qr);
+            const NetCost d = dense_cost(N, quads[k], (double)in.net_syn[b], std::max(cl, 1), stages);
+            pick[k] = cl && keep(d, items[k]);
+            cost.push_back(pick[k] ? d : items[k]);
             ctas += cost.back().cl;
         }
         return ctas;
     };
-    std::vector<uint8_t> pick, by_alone;
-    std::vector<NetCost> cost;
+    auto alone = [](const NetCost &d, const NetCost &i) { return d.alone <= 1.1 * i.alone; };
+    std::vector<uint8_t> pick, other;
     bool done = nets.empty();
     for (int f = PSST_MAX_CL; !done && f >= 1 && (long long)nets.size() <= sms; f /= 2)
-        done = choose(f, true, pick, cost) <= sms;
-    if (!done && choose(1, false, pick, cost) <= 4LL * sms) {
-        const double by_sm = step_time(cost, sms);
-        choose(1, true, by_alone, cost);
-        if (step_time(cost, sms) < by_sm) pick = by_alone;
+        done = choose(f, alone, pick) <= sms;
+    if (!done) {
+        choose(1, [](const NetCost &, const NetCost &) { return true; }, pick);
+        double best = 0.94 * step_time(cost, sms);
+        for (int by = 0; by < 2; ++by) {
+            if (by == 0) choose(1, [](const NetCost &d, const NetCost &i) { return d.sm <= 1.05 * i.sm; }, other);
+            else choose(1, alone, other);
+            const double t = step_time(cost, sms);
+            if (t < best) {
+                best = t;
+                pick = other;
+            }
+        }
     }
+    std::vector<uint8_t> dense((size_t)n_nets, 0);
     for (size_t k = 0; k < nets.size(); ++k) dense[nets[k]] = pick[k];
     return dense;
 }
@@ -939,7 +955,7 @@ int setup_cta(psst_net *h, const SmemCaps &caps, cudaError_t *err) {
     int sms = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e != cudaSuccess) return *err = e, cuda_fail(e, "device attributes");
-    const std::vector<uint8_t> dense = choose_dense(in, caps, sms);
+    const std::vector<uint8_t> dense = choose_dense(in, caps, sms, psst::method_stages(h->v));
     for (int b = 0; b < n_nets; ++b) {
         const int n0 = in.net_off[b], N = in.net_off[b + 1] - n0;
         if (in.net_syn[b] == 0) {  // independent neurons: no size class, no barrier

@@ -27,7 +27,7 @@ def _batch(n, p, nets, seed):
 # networks, neurons, connectivity, dense rows expected
 CASES = {"many, 1%": (200, 300, 0.01, False), "many, 10%": (200, 200, 0.1, False), "many, 45%": (170, 150, 0.45, True),
          "many small": (400, 24, 0.1, True), "few, 1%": (100, 300, 0.01, False), "alone, 10%": (1, 300, 0.1, True),
-         "alone, 1%": (1, 500, 0.01, False)}
+         "alone, 1%": (1, 500, 0.01, True)}
 
 
 @pytest.mark.parametrize("case", list(CASES))
