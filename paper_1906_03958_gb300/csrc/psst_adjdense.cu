@@ -34,7 +34,7 @@
 // memory per step (psst_adjoint.cu, kept for larger networks, duplicated
 // synapses and per-synapse gates).  Adjoint of 200 steps, us per step, before /
 // now: 64 lobes of 120 neurons 20 / 7.6, one of 37 neurons 14 / 3.6; with the
-// forward, 8617 -> 2682 us per pass and (300 steps) 6461 -> 2106.
+// forward, 8565 -> 2730 us per pass and (300 steps) 6497 -> 2110.
 #include <cuda_runtime.h>
 
 #include <type_traits>
